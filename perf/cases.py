@@ -118,8 +118,8 @@ def draw(rng):
     while True:
         # a chain or a ring of any length in the range, or a rectangle
         lo, hi = {"run_chain8": (4, 24), "run_chain64": (24, 64), "run_chain64_rbm": (6, 64),
-                  "sample_square10": (6, 160), "sample_chain64_rbm": (6, 64), "estimators_ring160": (8, 160), "observables_square10": (8, 128),
-                  "build_ring100": (10, 160), "solve_ring160": (10, 160), "snr_ring100": (8, 100),
+                  "sample_square10": (6, 160), "sample_chain64_rbm": (6, 64),
+                  "estimators_ring160": (8, 160), "observables_square10": (8, 128), "build_ring100": (10, 160), "solve_ring160": (10, 160), "snr_ring100": (8, 100),
                   "linear_square10": (24, 100), "linear_chain32_fp64": (5, 36)}[name]
         c["lx"], c["ly"] = _log_int(rng, lo, hi), 1
         if not c["pbc"] and rng.random() < 0.3:
