@@ -60,40 +60,37 @@ __global__ void __launch_bounds__(SAMP_THREADS, 1) sample_jastrow_kernel(
     unsigned char* tab = smp + 3 * (size_t)n * sizeof(float);  // [n][L] rows
     const double2* th = theta + (size_t)t * P;
 
-    // per site: largest group sum of |Re eta|, R_j (a warp per site, a lane per group)
-    {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        for (int j = warp; j < n; j += TPB >> 5) {
-            float mx = 0.f, tot = 0.f;
-            bool bad = false;
-            for (int g = lane; g < L; g += 32) {
-                float s = 0.f;
-                for (int k = g * B; k < min(n, (g + 1) * B); ++k)
-                    if (k != j) s += fabsf((float)th[n + pair_index(min(j, k), max(j, k), n)].x);
-                mx = fmaxf(mx, s);
-                bad = bad || !isfinite(s);
-                tot += s;
-            }
+    // per site: largest group sum of |Re eta|, R_j (a thread per site and group)
+    const int L1 = L * n;
+    for (int j = threadIdx.x; j < n; j += TPB) csc[j] = cg[j] = 0.f;
+    __syncthreads();
+#pragma unroll 2
+    for (int e = threadIdx.x; e < L1; e += TPB) {
+        const int g = e / n, j = e - g * n;
+        float q = 0.f;
 #pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-                tot += __shfl_xor_sync(0xffffffffu, tot, off);
-            }
-            bad = __any_sync(0xffffffffu, bad);
-            if (lane == 0) {
-                const float a = (float)th[j].x;
-                const float sc = mx * (1.000001f / 32767.f), R = (tot + fabsf(a)) * 1.00001f;
-                ca[j] = a;
-                csc[j] = bad ? 0.f : sc;
-                // 4.4 = 4 with a tenth to spare; 12 2^-24 R_j: the FP32 roundings
-                cg[j] = bad ? INFINITY : 4.4f * (0.52f * (float)L * sc + 7.2e-7f * R) + 1e-6f;
-            }
+        for (int b = 0; b < B; ++b) {
+            const int k = g * B + b;
+            if (k < n && k != j) q += fabsf((float)th[n + pair_index(min(j, k), max(j, k), n)].x);
         }
+        // (non-negative floats order as their bits; a NaN is the largest of them)
+        atomicMax(reinterpret_cast<int*>(csc + j), __float_as_int(q));
+        atomicAdd(cg + j, q);
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += TPB) {
+        const float a = (float)th[j].x, mx = csc[j];
+        const float sc = mx * (1.000001f / 32767.f), R = (cg[j] + fabsf(a)) * 1.00001f;
+        const bool bad = !isfinite(R);
+        ca[j] = a;
+        csc[j] = bad ? 0.f : sc;
+        // 4.4 = 4 with a tenth to spare; 12 2^-24 R_j: the FP32 roundings
+        cg[j] = bad ? INFINITY : 4.4f * (0.52f * (float)L * sc + 7.2e-7f * R) + 1e-6f;
     }
     __syncthreads();
     // the table, a (group, site) row per thread: 2^B sums out of two halves
     const int JS = samp_site(B, L);
-    for (int e = threadIdx.x; e < L * n; e += TPB) {
+    for (int e = threadIdx.x; e < L1; e += TPB) {
         const int g = e / n, j = e - g * n;
         float q[B];
         const float inv = csc[j] > 0.f ? 1.f / csc[j] : 0.f;
@@ -249,7 +246,8 @@ cudaError_t launch_sample_jastrow(const otvmc_ansatz* an, const double2* theta, 
     // 32 warps per SM: one CTA where the table takes more than half of the shared memory, else
     // two of 512; smaller CTAs while the batch leaves SMs without one
     int tpb = smem > 113 * 1024 ? 1024 : 512;
-    while (tpb > 64 && (tpb / 2 >= ns || (long long)ntraj * ((ns + tpb - 1) / tpb) < 152)) tpb /= 2;
+    while (tpb > 64 && (tpb / 2 >= ns || (tpb > 128 && (long long)ntraj * ((ns + tpb - 1) / tpb) < 152)))
+        tpb /= 2;
     fn<<<dim3((ns + tpb - 1) / tpb, ntraj), tpb, smem, s>>>(theta, (int)an->P, n, W, ns, n_sweep, (uint32_t)seed,
                                                             (uint32_t)(seed >> 32), evtag, traj0, spins, accepted);
     count_launch();
