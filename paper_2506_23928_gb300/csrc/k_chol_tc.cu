@@ -36,6 +36,7 @@
 #include <mutex>
 #include <string>
 
+#include "chol_tile.cuh"
 #include "common.cuh"
 #include "tc_common.cuh"
 
@@ -292,8 +293,6 @@ __device__ __forceinline__ void store_L8(float* Lft, piece_t* Lbt, const LbLayou
     }
 }
 
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-
 __device__ __forceinline__ float dot4(float4 a, float4 b, float s) {
     return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, s))));
 }
@@ -338,129 +337,55 @@ __device__ __forceinline__ int reduce8_index(int lane) {
 //     L_ik = A_ik X_kk^T (i > k);   X_kj = X_kk W_kj (j < k)
 //     A_ij -= L_ik L_jk^T (k < j <= i);   W_ij -= L_ik X_kj (i > k, j <= k)
 // W starts as the identity, so that X is the block forward substitution of L X = I.  The tile
-// products are warp-level SIMT GEMMs on float4 shared-memory operands.  Warp 0 updates A_k+1,k+1
-// first and factors it at once, while the other warps finish the remaining updates of step k.
+// products are warp-level SIMT GEMMs on float4 shared-memory operands.  A_k+1,k+1 is updated first
+// (by four warps) and warp 0 factors it at once, while the others finish the updates of step k.
 // The forward substitution of the solve is fused in: the block's right-hand sides (D for the
 // first block, else the running residual that the panel kernels of earlier block columns left
-// behind) are multiplied by X here.  Rows and columns beyond nb are padded with the identity.
+// behind) are multiplied by X here.  Rows and columns beyond nb are padded with the identity, and
+// whole tiles beyond it are left out.
+// Bound: latency, four warp factors of 4,600 to 5,500 cycles and two short phases between them
+// (39,000 cycles), the loads (6,000) and the outputs (9,500).  64 trajectories a launch: 34 us (62
+// us with the warp factor unrolled, one warp per panel tile and loads through registers); 4
+// trajectories of 36 parameters: 19 us (41 us).
 constexpr int DIAG_THREADS = 256;
 constexpr int HB = 64;                      // half block
-constexpr int TB = 32;                      // tile of the block algorithm
 constexpr int DSD = NB + 4;                 // shared row of the 128-wide block (16-byte aligned)
 constexpr int DSX = HB + 4;                 // shared row of a 64-wide quarter of the inverse
 // The inverse is kept as its three nonzero 64 x 64 quarters X11, X21, X22 (X12 = 0), so that the
 // kernel's ~119 KB of shared memory leaves room for an update-kernel CTA on the same SM.
 constexpr int DIAG_SMEM = (NB * DSD + 3 * HB * DSX + 2 * NB) * (int)sizeof(float) + 16;
 
-// Factor the 32 x 32 tile at A (row stride lda; lower triangle read) into L (written in place,
-// zeros above the diagonal) and write X = L^-1 to X (row stride ldx, zeros above the diagonal).
-// One warp: lane i holds row i of both.  Step m: the pivot is broadcast, lanes i >= m scale
-// their entry of column m, lane m scales its row of X; column m of L and row m of X go to the
-// scratch (scr: 128 floats, two buffers alternating by step), and every lane i > m subtracts
-// L_im times them, reading the scratch four entries at a time.
-// Returns false (uniformly over the warp) on a pivot that is not finite or not above dmin.
-__device__ __noinline__ bool factor32(float* A, int lda, float* X, int ldx, float* scr, float dmin) {
-    const int lane = threadIdx.x & 31;
-    float a[TB], x[TB];
-#pragma unroll
-    for (int q = 0; q < TB / 4; ++q) {
-        const float4 v = ld4(A + lane * lda + 4 * q);
-        a[4 * q] = v.x;
-        a[4 * q + 1] = v.y;
-        a[4 * q + 2] = v.z;
-        a[4 * q + 3] = v.w;
-    }
-#pragma unroll
-    for (int j = 0; j < TB; ++j) {
-        if (j > lane) a[j] = 0.f;
-        x[j] = j == lane ? 1.f : 0.f;
-    }
-    bool ok = true;
-#pragma unroll
-    for (int m = 0; m < TB; ++m) {
-        float* col = scr + (m & 1) * 2 * TB;
-        float* xrow = col + TB;
-        const float d = __shfl_sync(0xffffffffu, a[m], m);
-        ok = ok && d > dmin && isfinite(d);
-        // a few ulps suffice here: the factor is refined against the exact matrix later
-        const float isd = rsqrtf(ok ? d : 1.f);
-        const float l = lane >= m ? a[m] * isd : 0.f;
-        a[m] = l;
-        col[lane] = l;
-        if (lane == m) {
-#pragma unroll
-            for (int j = 0; j <= m; ++j) x[j] *= isd;
-#pragma unroll
-            for (int q = 0; q <= m / 4; ++q)
-                *reinterpret_cast<float4*>(xrow + 4 * q) = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-        }
-        __syncwarp();
-        const float lu = lane > m ? l : 0.f;
-#pragma unroll
-        for (int q = (m + 1) / 4; q < TB / 4; ++q) {
-            const float4 c = ld4(col + 4 * q);
-            if (4 * q + 0 > m) a[4 * q + 0] = fmaf(-lu, c.x, a[4 * q + 0]);
-            if (4 * q + 1 > m) a[4 * q + 1] = fmaf(-lu, c.y, a[4 * q + 1]);
-            if (4 * q + 2 > m) a[4 * q + 2] = fmaf(-lu, c.z, a[4 * q + 2]);
-            if (4 * q + 3 > m) a[4 * q + 3] = fmaf(-lu, c.w, a[4 * q + 3]);
-        }
-#pragma unroll
-        for (int q = 0; q <= m / 4; ++q) {
-            const float4 r = ld4(xrow + 4 * q);
-            if (4 * q + 0 <= m) x[4 * q + 0] = fmaf(-lu, r.x, x[4 * q + 0]);
-            if (4 * q + 1 <= m) x[4 * q + 1] = fmaf(-lu, r.y, x[4 * q + 1]);
-            if (4 * q + 2 <= m) x[4 * q + 2] = fmaf(-lu, r.z, x[4 * q + 2]);
-            if (4 * q + 3 <= m) x[4 * q + 3] = fmaf(-lu, r.w, x[4 * q + 3]);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < TB / 4; ++q) {
-        float4 v, w;
-        v.x = 4 * q + 0 <= lane ? a[4 * q + 0] : 0.f;
-        v.y = 4 * q + 1 <= lane ? a[4 * q + 1] : 0.f;
-        v.z = 4 * q + 2 <= lane ? a[4 * q + 2] : 0.f;
-        v.w = 4 * q + 3 <= lane ? a[4 * q + 3] : 0.f;
-        w.x = x[4 * q];
-        w.y = x[4 * q + 1];
-        w.z = x[4 * q + 2];
-        w.w = x[4 * q + 3];
-        *reinterpret_cast<float4*>(A + lane * lda + 4 * q) = v;
-        *reinterpret_cast<float4*>(X + lane * ldx + 4 * q) = w;
-    }
-    __syncwarp();
-    return ok;
-}
-
-// 32 x 32 x 32 tile products of one warp on shared-memory operands (row strides lda, ldb
-// multiples of 4 and = 4 mod 32: conflict-free float4 rows).  Lane (g, c) = (lane / 4, lane % 4)
-// owns rows g + 8 a (a < 4).
-// NT: acc[a][b] = sum_m A[g + 8a][m] B[c + 4b][m]   (columns c + 4 b)
-__device__ __forceinline__ void tile_nt(const float* A, int lda, const float* B, int ldb, float (&acc)[4][8]) {
+// Products of one warp on 32-wide shared-memory tiles (row strides lda, ldb multiples of 4 and
+// = 4 mod 32: conflict-free float4 rows), lane (g, c) = (lane / 4, lane % 4).
+// NT: acc[a][b] = sum_m A[g + 8 (a0 + a)][m] B[c + 4 b][m], NA of the four row groups
+template <int NA>
+__device__ __forceinline__ void tile_nt(const float* A, int lda, const float* B, int ldb, int a0, float (&acc)[NA][8]) {
     const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int a = 0; a < NA; ++a)
 #pragma unroll
         for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
 #pragma unroll 2
     for (int m = 0; m < TB; m += 4) {
-        float4 av[4], bv[8];
+        float4 av[NA], bv[8];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) av[a] = ld4(A + (g + 8 * a) * lda + m);
+        for (int a = 0; a < NA; ++a) av[a] = ld4(A + (g + 8 * (a0 + a)) * lda + m);
 #pragma unroll
         for (int b = 0; b < 8; ++b) bv[b] = ld4(B + (c + 4 * b) * ldb + m);
 #pragma unroll
-        for (int a = 0; a < 4; ++a)
+        for (int a = 0; a < NA; ++a)
 #pragma unroll
             for (int b = 0; b < 8; ++b) acc[a][b] = dot4(av[a], bv[b], acc[a][b]);
     }
 }
-// NN: acc[a][b] = sum_m A[g + 8a][m] B[m][8c + b]   (columns 8 c + b)
-__device__ __forceinline__ void tile_nn(const float* A, int lda, const float* B, int ldb, float (&acc)[4][8]) {
+// NN: acc[a][b] = sum_m A[g + 8 a][m] B[m][j0 + CB c + b], 4 CB columns from j0 (CB = 4 or 8)
+template <int CB>
+__device__ __forceinline__ void tile_nn(const float* A, int lda, const float* B, int ldb, int j0, float (&acc)[4][CB]) {
     const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] = 0.f;
+        for (int b = 0; b < CB; ++b) acc[a][b] = 0.f;
 #pragma unroll 2
     for (int m = 0; m < TB; m += 4) {
         float4 av[4];
@@ -468,31 +393,44 @@ __device__ __forceinline__ void tile_nn(const float* A, int lda, const float* B,
         for (int a = 0; a < 4; ++a) av[a] = ld4(A + (g + 8 * a) * lda + m);
 #pragma unroll
         for (int mm = 0; mm < 4; ++mm) {
-            const float4 b0 = ld4(B + (m + mm) * ldb + 8 * c), b1 = ld4(B + (m + mm) * ldb + 8 * c + 4);
+            float bv[CB];
+#pragma unroll
+            for (int q = 0; q < CB / 4; ++q) {
+                const float4 v = ld4(B + (m + mm) * ldb + j0 + CB * c + 4 * q);
+                bv[4 * q] = v.x;
+                bv[4 * q + 1] = v.y;
+                bv[4 * q + 2] = v.z;
+                bv[4 * q + 3] = v.w;
+            }
 #pragma unroll
             for (int a = 0; a < 4; ++a) {
                 const float s = mm == 0 ? av[a].x : mm == 1 ? av[a].y : mm == 2 ? av[a].z : av[a].w;
-                acc[a][0] = fmaf(s, b0.x, acc[a][0]);
-                acc[a][1] = fmaf(s, b0.y, acc[a][1]);
-                acc[a][2] = fmaf(s, b0.z, acc[a][2]);
-                acc[a][3] = fmaf(s, b0.w, acc[a][3]);
-                acc[a][4] = fmaf(s, b1.x, acc[a][4]);
-                acc[a][5] = fmaf(s, b1.y, acc[a][5]);
-                acc[a][6] = fmaf(s, b1.z, acc[a][6]);
-                acc[a][7] = fmaf(s, b1.w, acc[a][7]);
+#pragma unroll
+                for (int b = 0; b < CB; ++b) acc[a][b] = fmaf(s, bv[b], acc[a][b]);
             }
         }
     }
 }
-// C = sgn * acc (set) or C -= acc (sub), in the column layout of tile_nt (nt) or tile_nn.
-template <bool NT>
-__device__ __forceinline__ void tile_store(float* C, int ldc, const float (&acc)[4][8], bool sub) {
+// C = acc (set) or C -= acc (sub), in the layout of tile_nt or tile_nn.
+template <int NA>
+__device__ __forceinline__ void store_nt(float* C, int ldc, int a0, const float (&acc)[NA][8], bool sub) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+#pragma unroll
+    for (int a = 0; a < NA; ++a)
+#pragma unroll
+        for (int b = 0; b < 8; ++b) {
+            float& dst = C[(g + 8 * (a0 + a)) * ldc + c + 4 * b];
+            dst = sub ? dst - acc[a][b] : acc[a][b];
+        }
+}
+template <int CB>
+__device__ __forceinline__ void store_nn(float* C, int ldc, int j0, const float (&acc)[4][CB], bool sub) {
     const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            float& dst = C[(g + 8 * a) * ldc + (NT ? c + 4 * b : 8 * c + b)];
+        for (int b = 0; b < CB; ++b) {
+            float& dst = C[(g + 8 * a) * ldc + j0 + CB * c + b];
             dst = sub ? dst - acc[a][b] : acc[a][b];
         }
 }
@@ -510,39 +448,51 @@ struct DiagTiles {
     }
 };
 
-// Phase "panel" of step k: job q < 3 - k is L_ik = A_ik X_kk^T with i = k + 1 + q; the others
-// X_kj = X_kk W_kj with j = q - (3 - k).  In place: each job owns its output tile.
-__device__ void diag_panel_job(const DiagTiles& T, int k, int q) {
-    float acc[4][8];
-    if (q < 3 - k) {
+// Phase "panel" of step k of nt tiles: tile q < nt - 1 - k is L_ik = A_ik X_kk^T with i = k + 1 + q;
+// the k others X_kj = X_kk W_kj with j = q - (nt - 1 - k).  Two warps per tile, in place: the first
+// kind split by rows, the second by columns (each half reads only what it overwrites).
+__device__ void diag_panel_job(const DiagTiles& T, int nt, int k, int q, int half) {
+    if (q < nt - 1 - k) {
+        float acc[2][8];
         float* Aik = T.a(k + 1 + q, k);
-        tile_nt(Aik, DSD, T.x(k, k), DSX, acc);
+        tile_nt<2>(Aik, DSD, T.x(k, k), DSX, 2 * half, acc);
         __syncwarp();
-        tile_store<true>(Aik, DSD, acc, false);
+        store_nt<2>(Aik, DSD, 2 * half, acc, false);
     } else {
-        float* Wkj = T.x(k, q - (3 - k));
-        tile_nn(T.x(k, k), DSX, Wkj, DSX, acc);
+        float acc[4][4];
+        float* Wkj = T.x(k, q - (nt - 1 - k));
+        tile_nn<4>(T.x(k, k), DSX, Wkj, DSX, 16 * half, acc);
         __syncwarp();
-        tile_store<false>(Wkj, DSX, acc, false);
+        store_nn<4>(Wkj, DSX, 16 * half, acc, false);
     }
     __syncwarp();
 }
-// Phase "update" of step k: the (3-k)(4-k)/2 tiles A_ij -= L_ik L_jk^T (k < j <= i) and the
-// (3-k)(k+1) tiles W_ij -= L_ik X_kj (i > k, j <= k), numbered A tiles first, row by row.
-__device__ int diag_update_jobs(int k) { return (3 - k) * (4 - k) / 2 + (3 - k) * (k + 1); }
-__device__ void diag_update_job(const DiagTiles& T, int k, int q) {
-    float acc[4][8];
-    const int nA = (3 - k) * (4 - k) / 2;
+// Phase "update" of step k, r = nt - 1 - k tile rows below: the r (r + 1) / 2 tiles A_ij -= L_ik L_jk^T
+// (k < j <= i) and the r (k + 1) tiles W_ij -= L_ik X_kj (i > k, j <= k), A tiles first, row by row.
+// Job 0, the next diagonal tile, is taken by four warps (a row group each) before the others.
+__device__ int diag_update_jobs(int nt, int k) {
+    const int r = nt - 1 - k;
+    return r * (r + 1) / 2 + r * (k + 1);
+}
+__device__ void diag_next_tile(const DiagTiles& T, int k, int a0) {
+    float acc[1][8];
+    tile_nt<1>(T.a(k + 1, k), DSD, T.a(k + 1, k), DSD, a0, acc);
+    store_nt<1>(T.a(k + 1, k + 1), DSD, a0, acc, true);
+}
+__device__ void diag_update_job(const DiagTiles& T, int nt, int k, int q) {
+    const int nA = (nt - 1 - k) * (nt - k) / 2;
     if (q < nA) {
+        float acc[4][8];
         int i = k + 1, r = q;
         while (r > i - k - 1) { r -= i - k; ++i; }
         const int j = k + 1 + r;
-        tile_nt(T.a(i, k), DSD, T.a(j, k), DSD, acc);
-        tile_store<true>(T.a(i, j), DSD, acc, true);
+        tile_nt<4>(T.a(i, k), DSD, T.a(j, k), DSD, 0, acc);
+        store_nt<4>(T.a(i, j), DSD, 0, acc, true);
     } else {
+        float acc[4][8];
         const int r = q - nA, i = k + 1 + r / (k + 1), j = r % (k + 1);
-        tile_nn(T.a(i, k), DSD, T.x(k, j), DSX, acc);
-        tile_store<false>(T.x(i, j), DSX, acc, true);
+        tile_nn<8>(T.a(i, k), DSD, T.x(k, j), DSX, 0, acc);
+        store_nn<8>(T.x(i, j), DSX, 0, acc, true);
     }
     __syncwarp();
 }
@@ -570,6 +520,7 @@ __global__ void __launch_bounds__(DIAG_THREADS) chol_diag_kernel(int t0, int P, 
     const DiagTiles T{A, X11, X21, X22};
     const int tid = threadIdx.x, warp = tid >> 5;
     const int nb = min(NB, P - jb);
+    const int nt = (nb + TB - 1) / TB;  // tiles of the last, smaller block: the padding stays untouched
     float* yt = yv + (size_t)t * 2 * P;
     const double2* Dt = D + (size_t)t * P;
     const float sc = inv_s[t];
@@ -590,13 +541,27 @@ __global__ void __launch_bounds__(DIAG_THREADS) chol_diag_kernel(int t0, int P, 
             yt[k] = (float)d.x * sc;
             yt[P + k] = (float)d.y * sc;
         }
-    // the lower block (with the diagonal), identity padding beyond nb; lanes along rows i.
-    // Loads are issued in batches of 32 per thread before any of them is used.
-    {
+    // the lower block (with the diagonal), identity padding beyond nb; lanes along rows i.  Later
+    // block columns come from the update kernel by asynchronous copies, all in flight at once; the
+    // first from the Gram counts, 32 loads per thread issued before any of them is used.
+    if (jb > 0) {
+        const float* Pt = Pn + (size_t)t * NB * P + jb;
+#pragma unroll 8
+        for (int e = tid; e < NB * NB; e += DIAG_THREADS) {
+            const int c = e >> 7, i = e & (NB - 1);
+            float* dst = A + i * DSD + c;
+            if (i < nb && c <= i)  // c <= i < nb
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)),
+                             "l"(Pt + (size_t)c * P + i));
+            else
+                *dst = i == c ? 1.f : 0.f;
+        }
+        asm volatile("cp.async.wait_all;" ::: "memory");
+    } else {
         const float* Gt = G + (size_t)t * P * P;
         const float inv_ns = 1.0f / (float)ns;
         float* obs = X11;  // the block's column means (first block column only), X not yet in use
-        if (jb == 0 && tid < NB) obs[tid] = tid < nb ? (float)obar[(size_t)t * P + tid] : 0.f;
+        if (tid < NB) obs[tid] = tid < nb ? (float)obar[(size_t)t * P + tid] : 0.f;
         __syncthreads();
 #pragma unroll 1
         for (int base = 0; base < NB * NB; base += 32 * DIAG_THREADS) {
@@ -605,8 +570,7 @@ __global__ void __launch_bounds__(DIAG_THREADS) chol_diag_kernel(int t0, int P, 
             for (int q = 0; q < 32; ++q) {
                 const int e = base + tid + DIAG_THREADS * q, c = e >> 7, i = e & (NB - 1);
                 float x = 0.f;
-                if (i < nb && c < nb && c <= i)
-                    x = jb == 0 ? Gt[(size_t)c * P + i] : Pn[((size_t)t * NB + c) * P + jb + i];
+                if (i < nb && c < nb && c <= i) x = Gt[(size_t)c * P + i];
                 v[q] = x;
             }
 #pragma unroll
@@ -614,49 +578,44 @@ __global__ void __launch_bounds__(DIAG_THREADS) chol_diag_kernel(int t0, int P, 
                 const int e = base + tid + DIAG_THREADS * q, c = e >> 7, i = e & (NB - 1);
                 float x = i == c ? 1.f : 0.f;
                 if (i < nb && c < nb && c <= i) {
-                    x = v[q];
-                    if (jb == 0) {
-                        x = x * inv_ns - obs[i] * obs[c];
-                        if (i == c) x += eps;
-                        x *= sc;
-                    }
+                    x = v[q] * inv_ns - obs[i] * obs[c];
+                    if (i == c) x += eps;
+                    x *= sc;
                 }
                 A[i * DSD + c] = x;
             }
         }
     }
     __syncthreads();
-    // W: zero below the diagonal tiles (the diagonal tiles are written by factor32)
-    if (warp == 0) {
-        const bool ok = factor32(T.a(0, 0), DSD, T.x(0, 0), DSX, fscr, dmin);
-        if (tid == 0) pivots_ok = ok;
-    } else {
-        for (int e = tid - 32; e < 6 * TB * TB / 4; e += DIAG_THREADS - 32) {
-            const int q = e / (TB * TB / 4), r = (e >> 3) & (TB - 1), c4 = e & 7;
-            const int i = q == 0 ? 1 : q < 3 ? 2 : 3;
-            const int j = q == 0 ? 0 : q == 1 ? 0 : q == 2 ? 1 : q == 3 ? 0 : q == 4 ? 1 : 2;
-            *reinterpret_cast<float4*>(T.x(i, j) + r * DSX + 4 * c4) = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
-    __syncthreads();
+    // Step k: warp 0 factors diagonal tile k while six others (not warp 4, which shares warp 0's
+    // scheduler) finish the updates of step k - 1, or set W to zero below the diagonal tiles before
+    // the first; then all do the panel, and four warps the next diagonal tile.
+    const int job_warp = warp < 4 ? warp - 1 : warp - 2;
 #pragma unroll 1
-    for (int k = 0; k < 4; ++k) {
+    for (int k = 0; k < nt; ++k) {
+        if (warp == 0) {
+            const bool ok = factor32(T.a(k, k), DSD, T.x(k, k), DSX, fscr, dmin);
+            if (tid == 0) pivots_ok = ok;
+        } else if (warp != 4 && k > 0) {
+            const int nj = diag_update_jobs(nt, k - 1);
+            for (int q = 1 + job_warp; q < nj; q += 6) diag_update_job(T, nt, k - 1, q);
+        } else if (k == 0) {
+            for (int e = tid - 32; e < 6 * TB * TB / 4; e += DIAG_THREADS - 32) {
+                const int q = e / (TB * TB / 4), r = (e >> 3) & (TB - 1), c4 = e & 7;
+                const int i = q == 0 ? 1 : q < 3 ? 2 : 3;
+                const int j = q == 0 ? 0 : q == 1 ? 0 : q == 2 ? 1 : q == 3 ? 0 : q == 4 ? 1 : 2;
+                *reinterpret_cast<float4*>(T.x(i, j) + r * DSX + 4 * c4) = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+        __syncthreads();
         if (!pivots_ok) {  // uniform: read after a barrier
             if (tid == 0) fail[t] = 1;
             return;
         }
-        if (warp < 3) diag_panel_job(T, k, warp);
+        if (warp < 2 * (nt - 1)) diag_panel_job(T, nt, k, warp >> 1, warp & 1);
         __syncthreads();
-        if (k == 3) break;
-        // warp 0: the next diagonal tile's update (job 0), then its factor; the others the rest
-        const int nj = diag_update_jobs(k);
-        if (warp == 0) {
-            diag_update_job(T, k, 0);
-            const bool ok = factor32(T.a(k + 1, k + 1), DSD, T.x(k + 1, k + 1), DSX, fscr, dmin);
-            if (tid == 0) pivots_ok = ok;
-        } else {
-            for (int q = warp; q < nj; q += DIAG_THREADS / 32 - 1) diag_update_job(T, k, q);
-        }
+        if (k == nt - 1) break;
+        if (warp < 4) diag_next_tile(T, k, warp);
         __syncthreads();
     }
     // outputs: L (FP32 and FP16 pieces), X (padded rows / columns zero), y_b = X rhs
