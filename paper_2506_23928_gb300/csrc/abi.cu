@@ -135,6 +135,15 @@ static size_t obuf_bytes(const otvmc_ansatz* a, int T, int ns, int precision) {
     return (size_t)T * (a->P + D_XROWS) * o_pitch(ns) + 256;  // E4M3 O and its extra rows
 }
 
+// FP64 path: where the tensor-core Gram counts (FP32, [T][P][P]) start in the buffer of the FP64
+// O, behind the E4M3 O; 0 when the two do not fit (more than about 1.7 parameters per sample) or
+// the counts leave FP32's whole numbers.
+static size_t gram_in_obuf(const otvmc_ansatz* a, int T, int ns) {
+    const size_t o = ((size_t)T * a->P * o_pitch(ns) + 255) & ~(size_t)255;
+    const size_t g = (size_t)T * a->P * a->P * sizeof(float);
+    return ns < (1 << 24) && o + g <= obuf_bytes(a, T, ns, OTVMC_PREC_FP64) ? o : 0;
+}
+
 static bool valid_ansatz(const otvmc_ansatz* a) { return a != nullptr && a->model != nullptr && a->P > 0; }
 
 static otvmc_status check_batch(const otvmc_ansatz* a, int ntraj, int ns) {
@@ -599,10 +608,22 @@ static otvmc_status run_build(const otvmc_ansatz* a, const uint64_t* spins, cons
     CK(launch_vquant(T, ns, v, b, s), "vquant launch");
     if (precision == OTVMC_PREC_FP64) {
         CK(launch_D_fixed_jastrow(a, spins, T, ns, b, obar, D, s), "D launch");
-        double* Oc = (double*)obuf;
-        CK(launch_obuild_f64_jastrow(a, spins, T, ns, obar, Oc, s), "obuild f64 launch");
-        CK(launch_syrk_f64(T, P, ns, Oc, S, s), "syrk launch");
-        CK(launch_gemv_D_f64(T, P, ns, Oc, v, b, D, s), "gemv launch");
+        CK(launch_D_f64(a, spins, T, ns, obar, v, b, D, s), "D launch");
+        const size_t gram_b = gram_in_obuf(a, T, ns);
+        if (gram_b) {
+            // the Gram counts are whole numbers, exact from the tensor cores: S from them is
+            // rounded twice, where the FP64 sums of centred products round ns times
+            uint8_t* Ot = (uint8_t*)obuf;
+            float* Gc = (float*)((char*)obuf + gram_b);
+            CK(launch_obuild_f8_jastrow(a, spins, T, ns, nullptr, Ot, s), "obuild launch");
+            CK(launch_gram_tc(T, P, P, ns, o_pitch(ns), Ot, a->tiles_d, a->ntiles, Gc, nullptr, status, s),
+               "gram launch");
+            CK(launch_S_counts(T, P, ns, Gc, obar, S, s), "S launch");
+        } else {
+            double* Oc = (double*)obuf;
+            CK(launch_obuild_f64_jastrow(a, spins, T, ns, obar, Oc, s), "obuild f64 launch");
+            CK(launch_syrk_f64(T, P, ns, Oc, S, s), "syrk launch");
+        }
     } else {
         // D and obar from the Gram pass (the digits of q as extra rows of O) while the digit
         // sums stay exact in FP32; else by the integer sums

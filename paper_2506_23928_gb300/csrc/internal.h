@@ -177,8 +177,9 @@ cudaError_t launch_obuild_f8_jastrow(const otvmc_ansatz* a, const uint64_t* spin
 cudaError_t launch_obuild_f64_jastrow(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns,
                                       const double* obar, double* Oc, cudaStream_t s);
 cudaError_t launch_syrk_f64(int ntraj, int P, int ns, const double* Oc, double* S, cudaStream_t s);
-cudaError_t launch_gemv_D_f64(int ntraj, int P, int ns, const double* Oc, const double2* v, const EvalBufs& b,
-                              double2* D, cudaStream_t s);
+cudaError_t launch_D_f64(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const double* obar,
+                         const double2* v, const EvalBufs& b, double2* D, cudaStream_t s);
+cudaError_t launch_S_counts(int ntraj, int P, int ns, const float* G, const double* obar, double* S, cudaStream_t s);
 std::vector<int2> gram_tiles(int P);
 std::vector<int2> gram_tiles_x(int P, int PC);
 // G (P x P, upper) from the E4M3 operand Ot [ntraj][rows][pitch] (pitch a multiple of 16, the

@@ -383,20 +383,29 @@ cudaError_t launch_syrk_f64(int ntraj, int P, int ns, const double* Oc, double* 
     return launch_syrk_f64_scaled(ntraj, P, ns, 1.0 / ns, Oc, S, s);
 }
 
-// D_k = sum_x Oc[k][x] (v(x) - vbar) / ns, FP64: one warp per parameter.
-__global__ void __launch_bounds__(256) gemv_D_f64_kernel(int P, int ns, const double* __restrict__ Oc,
-                                                         const double2* __restrict__ v,
-                                                         const double* __restrict__ vinfo, double2* __restrict__ D) {
+// D_k = sum_x (O_xk - obar_k) (v(x) - vbar) / ns, FP64: one warp per parameter, the signs from
+// the spins.
+__global__ void __launch_bounds__(256) D_f64_kernel(int n, int W, int P, int ns, const uint64_t* __restrict__ spins,
+                                                    const int* __restrict__ pairs, const double* __restrict__ obar,
+                                                    const double2* __restrict__ v, const double* __restrict__ vinfo,
+                                                    double2* __restrict__ D) {
     const int t = blockIdx.y;
     const int k = blockIdx.x * 8 + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;
     if (k >= P) return;
     const double mr = vinfo[4 * t], mi = vinfo[4 * t + 1];
-    const double* o = Oc + ((size_t)t * P + k) * ns;
+    const double ob = obar[(size_t)t * P + k];
+    const double up = 1.0 - ob, dn = -1.0 - ob;
+    // O = +1 where the bits of j and l agree (a single site: where its own bit is set)
+    const int j = k < n ? k : pairs[2 * (k - n)], l = k < n ? -1 : pairs[2 * (k - n) + 1];
+    const uint64_t* sp = spins + (size_t)t * ns * W;
     const double2* vv = v + (size_t)t * ns;
     double ar = 0.0, ai = 0.0;
+#pragma unroll 4
     for (int x = lane; x < ns; x += 32) {
-        const double c = o[x];
+        uint64_t b = sp[(size_t)x * W + (j >> 6)] >> (j & 63);
+        if (l >= 0) b = ~(b ^ (sp[(size_t)x * W + (l >> 6)] >> (l & 63)));
+        const double c = (b & 1ull) ? up : dn;
         ar = fma(c, vv[x].x - mr, ar);
         ai = fma(c, vv[x].y - mi, ai);
     }
@@ -408,11 +417,61 @@ __global__ void __launch_bounds__(256) gemv_D_f64_kernel(int P, int ns, const do
     if (lane == 0) D[(size_t)t * P + k] = make_double2(ar / ns, ai / ns);
 }
 
-cudaError_t launch_gemv_D_f64(int ntraj, int P, int ns, const double* Oc, const double2* v, const EvalBufs& b,
-                              double2* D, cudaStream_t s) {
+cudaError_t launch_D_f64(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const double* obar,
+                         const double2* v, const EvalBufs& b, double2* D, cudaStream_t s) {
     ProfScope prof_(OTVMC_K_D, s);
-    dim3 grid((P + 7) / 8, ntraj);
-    gemv_D_f64_kernel<<<grid, 256, 0, s>>>(P, ns, Oc, v, b.vinfo, D);
+    const int n = a->n, W = (n + 63) / 64, P = (int)a->P;
+    D_f64_kernel<<<dim3((P + 7) / 8, ntraj), 256, 0, s>>>(n, W, P, ns, spins, a->pairs_d, obar, v, b.vinfo, D);
+    count_launch();
+    return cudaGetLastError();
+}
+
+// S = G / ns - c c^T / ns^2 (full, FP64) from the exact counts G_ij = sum_x O_i O_j of the upper
+// triangle and c_i = sum_x O_i (= ns obar_i): (ns G_ij - c_i c_j) is formed exactly in 64-bit
+// integers (below 2^62 while ns |O|^2 < 2^31), so each entry is rounded only when it is converted
+// and when it is divided by ns^2.  One 32 x 32 tile of the upper triangle per CTA, its mirror
+// image written through shared memory.
+template <typename TG>
+__global__ void __launch_bounds__(256) S_counts_kernel(int P, int ns, const TG* __restrict__ G,
+                                                       const double* __restrict__ obar, double* __restrict__ S) {
+    constexpr int B = 32;
+    __shared__ double tile[B][B + 1];
+    __shared__ long long ci[B], cj[B];
+    const int t = blockIdx.y;
+    int J = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+    while ((J + 1) * (J + 2) / 2 <= (int)blockIdx.x) ++J;
+    while (J * (J + 1) / 2 > (int)blockIdx.x) --J;
+    const int I = blockIdx.x - J * (J + 1) / 2;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const double* ob = obar + (size_t)t * P;
+    if (threadIdx.x < B) ci[tx] = I * B + tx < P ? __double2ll_rn(ob[I * B + tx] * ns) : 0ll;
+    else if (threadIdx.x < 2 * B) cj[tx] = J * B + tx < P ? __double2ll_rn(ob[J * B + tx] * ns) : 0ll;
+    __syncthreads();
+    const TG* Gt = G + (size_t)t * P * P;
+    double* St = S + (size_t)t * P * P;
+    const double den = (double)ns * (double)ns;
+#pragma unroll
+    for (int r = ty; r < B; r += 8) {
+        const int i = I * B + r, j = J * B + tx;
+        double v = 0.0;
+        if (i < P && j < P && i <= j) {
+            v = (double)((long long)Gt[(size_t)i * P + j] * ns - ci[r] * cj[tx]) / den;
+            St[(size_t)i * P + j] = v;
+        }
+        tile[r][tx] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = ty; r < B; r += 8) {
+        const int j = J * B + r, i = I * B + tx;  // entry (j, i), i < j
+        if (i < P && j < P && i < j) St[(size_t)j * P + i] = tile[tx][r];
+    }
+}
+
+cudaError_t launch_S_counts(int ntraj, int P, int ns, const float* G, const double* obar, double* S, cudaStream_t s) {
+    ProfScope prof_(OTVMC_K_SYRK, s);
+    const int nt = (P + 31) / 32;
+    S_counts_kernel<float><<<dim3(nt * (nt + 1) / 2, ntraj), 256, 0, s>>>(P, ns, G, obar, S);
     count_launch();
     return cudaGetLastError();
 }
