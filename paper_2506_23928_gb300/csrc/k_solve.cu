@@ -7,7 +7,8 @@
 // block with one warp, and solve the panel below it.  The right-hand side is complex and
 // S real (Jastrow), so the real and imaginary parts are two right-hand sides.
 //
-// precision FP64: S given in full FP64, FP64 factor and solves.
+// precision FP64: S given in full FP64, FP64 factor and solves; from P = 48 only for the
+// trajectories that the FP32 factorization with FP64 refinement (k_solve_ref.cu) leaves.
 // precision MIXED: S = G / ns - obar obar^T from the exact Gram counts; FP32 factor and
 // solves, then `refine` steps of iterative refinement x += solve(D - (S + eps I) x) with the
 // residual formed in FP64 from G and obar.
@@ -365,6 +366,11 @@ __global__ void __launch_bounds__(256, 1) chol_solve_kernel(int P, int ns, doubl
     if (tid == 0 && shift_used) shift_used[t] = eps;
 }
 
+// FP32 factorization refined to FP64 (k_solve_ref.cu)
+bool solve_ref_ok(int P);
+cudaError_t launch_solve_ref(int ntraj, int P, double eps, const double* S, const double2* D, double2* delta,
+                             double* shift_used, double* Lws, double* xws, int* flags, cudaStream_t s);
+
 size_t chol_tc_ws_bytes(int ntraj, int P);
 cudaError_t launch_chol_tc(int ntraj, int P, int ns, double eps, const float* G, const double* obar,
                            const double2* D, double2* delta, double* shift_used, void* ws, int refine_iters,
@@ -372,7 +378,8 @@ cudaError_t launch_chol_tc(int ntraj, int P, int ns, double eps, const float* G,
 
 size_t chol_ws_bytes(int ntraj, int P, int precision) {
     if (precision != OTVMC_PREC_FP64) return chol_tc_ws_bytes(ntraj, P);
-    return (size_t)ntraj * ((size_t)P * P * 8 + 2 * (size_t)P * 8 + 4 * (size_t)P * 8) + 3 * 256;
+    // factor, right-hand sides, solution and residual, and a flag per trajectory
+    return (size_t)ntraj * ((size_t)P * P * 8 + 2 * (size_t)P * 8 + 4 * (size_t)P * 8 + 4) + 4 * 256;
 }
 
 cudaError_t launch_chol_solve_masked(int ntraj, int P, int ns, double eps, const float* G, const double* obar,
@@ -402,10 +409,18 @@ cudaError_t launch_chol_solve(int ntraj, int P, int ns, int precision, double ep
     void* L = take((size_t)ntraj * P * P * 8);
     void* y = take((size_t)ntraj * 2 * P * 8);
     double* x = (double*)take((size_t)ntraj * 4 * P * 8);
+    // FP32 factor and FP64 refinement first; the FP64 factorization then takes the trajectories
+    // that it left (their flags set), and all of them below the sizes it is built for
+    int* flags = nullptr;
+    if (solve_ref_ok(P)) {
+        flags = (int*)take((size_t)ntraj * 4);
+        const cudaError_t e = launch_solve_ref(ntraj, P, eps, S, D, delta, shift_used, (double*)L, x, flags, s);
+        if (e != cudaSuccess) return e;
+    }
     const int smem = (int)sizeof(SolveSmem<double>);
     cudaFuncSetAttribute(chol_solve_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     chol_solve_kernel<double, false><<<ntraj, 256, smem, s>>>(P, ns, eps, 0, S, G, obar, D, delta, shift_used,
-                                                              (double*)L, (size_t)P * P, (double*)y, x, nullptr,
+                                                              (double*)L, (size_t)P * P, (double*)y, x, flags,
                                                               status);
     count_launch();
     return cudaGetLastError();
