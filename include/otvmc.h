@@ -298,13 +298,12 @@ OTVMC_API otvmc_status otvmc_solve_step(const otvmc_ansatz* ansatz, int ntraj, i
  *   SNR_k = |rho_k| / sqrt(Var_x Q_k / ns),
  *   f_k = 1 / (1 + (snr_thresh / SNR_k)^6) * 1 / (1 + (eps_svd lambda_max / lambda_k)^6),
  *   delta = V diag(f_k / lambda_k) rho, eigenvalues lambda_k <= 0 dropped.
- * Jastrow and tied Jastrow ansaetze, one CTA per trajectory, FP64 throughout.  P <= 96: a
- * cyclic Jacobi eigen-decomposition in shared memory.  Larger P (up to what the shared memory
- * of one CTA holds for the tridiagonal and a chunk of samples, about 3000): Householder
- * tridiagonalisation of a copy of S in the workspace, the eigenvectors formed explicitly and
- * refined by the implicit QL iteration (shift from the leading 2 x 2 block), then one pass over
- * the samples; this costs O(P^3) FP64 work per trajectory for the decomposition and
- * O(ns P^2) for the pass.  Inputs: S_d [ntraj][P][P] full FP64 S (otvmc_build_S_F), obar_d
+ * Jastrow and tied Jastrow ansaetze, FP64 throughout.  P <= 96: a cyclic Jacobi
+ * eigen-decomposition in shared memory, one CTA per trajectory.  Larger P (up to about 3000):
+ * Householder tridiagonalisation of a copy of S in the workspace, the eigenvectors formed
+ * explicitly and refined by the implicit QL iteration (shift from the leading 2 x 2 block), and
+ * Var_x Q_k from M = sum_x |v_c|^2 O_c O_c^T (exact integer sums, |v_c|^2 to 46 bits of its largest
+ * value) as v_k^T M v_k; this costs O(P^3) FP64 work per trajectory and O(ns P^2) integer work.  Inputs: S_d [ntraj][P][P] full FP64 S (otvmc_build_S_F), obar_d
  * [ntraj][P], spins_d [ntraj][ns][W], v_d [ntraj][ns] double2 (otvmc_local_estimators), D_d
  * [ntraj][P] double2.  work_bytes >= otvmc_snr_workspace_bytes(ansatz, ntraj) (256 bytes of
  * status for P <= 96, plus 2 P^2 doubles per trajectory beyond).  Outputs: delta_d [ntraj][P]
@@ -355,9 +354,7 @@ OTVMC_API otvmc_status otvmc_ensemble(const double* moments_h, int ntraj, int n_
  * moments_d (may be NULL when measure_every = 0): [n_meas][ntraj][9] with one row per
  * measured step (steps i with i % measure_every == 0, from the predictor samples at
  * theta_i) plus, if measure_final, one row at the final time.  With OTVMC_REG_SNR the solve is
- * otvmc_solve_snr's filter; on the mixed path its pass over the samples (beyond P = 96) projects
- * in FP32 (the variances that set the filter to about 1e-6 relative).  Synchronises and returns
- * the device status at the end.  work_bytes >= otvmc_run_workspace_bytes(...). */
+ * otvmc_solve_snr's filter.  Synchronises and returns the device status at the end.  work_bytes >= otvmc_run_workspace_bytes(...). */
 typedef struct otvmc_run_desc {
     int ntraj;
     int traj0;

@@ -409,6 +409,7 @@ otvmc_status otvmc_ansatz_create_lj(const otvmc_model* model, int d, int pbc, ot
                 gpair.push_back(pidx(j, k));
                 off.push_back((int)gpair.size());
             }
+    const int nfree = (int)off.size() - 1;
     for (int D = d + 1; D < n; ++D) {
         const size_t before = gpair.size();
         for (int j = 0; j < n; ++j)
@@ -427,7 +428,11 @@ otvmc_status otvmc_ansatz_create_lj(const otvmc_model* model, int d, int pbc, ot
     a->lj_d = d;
     a->lj_pbc = pbc;
     a->ngroups = (int)off.size() - 1;
+    a->nfree = nfree;
     a->P = (int64_t)n + a->ngroups;
+    const int rows = lj_operand_rows(a);
+    const std::vector<int2> tiles = gram_tiles_x(rows, rows + D_XROWS);
+    a->ntiles = (int)tiles.size();
     bool ok = cudaMalloc(&a->grp_off_d, sizeof(int) * off.size()) == cudaSuccess &&
               cudaMemcpy(a->grp_off_d, off.data(), sizeof(int) * off.size(), cudaMemcpyHostToDevice) == cudaSuccess;
     if (ok && !gpair.empty())
@@ -436,6 +441,8 @@ otvmc_status otvmc_ansatz_create_lj(const otvmc_model* model, int d, int pbc, ot
                  cudaSuccess &&
              cudaMalloc(&a->pair_grp_d, sizeof(int) * pgrp.size()) == cudaSuccess &&
              cudaMemcpy(a->pair_grp_d, pgrp.data(), sizeof(int) * pgrp.size(), cudaMemcpyHostToDevice) == cudaSuccess;
+    ok = ok && cudaMalloc(&a->tiles_d, sizeof(int2) * tiles.size()) == cudaSuccess &&
+         cudaMemcpy(a->tiles_d, tiles.data(), sizeof(int2) * tiles.size(), cudaMemcpyHostToDevice) == cudaSuccess;
     if (!ok) {
         otvmc_ansatz_destroy(a);
         return fail(OTVMC_ERR_OOM, "device allocation for the ansatz failed");
@@ -674,7 +681,7 @@ otvmc_status otvmc_build_S_F(const otvmc_ansatz* a, const double* theta_d, const
         cudaStream_t s = (cudaStream_t)stream;
         CK(launch_vpart(ntraj, ns, (const double2*)v_d, b, s), "vpart launch");
         CK(launch_vquant(ntraj, ns, (const double2*)v_d, b, s), "vquant launch");
-        CK(launch_lj_build(a, spins_d, ntraj, ns, b, ws, S_d, obar, (double2*)D_d, s), "tied build launch");
+        CK(launch_lj_build(a, spins_d, ntraj, ns, b, ws, S_d, obar, (double2*)D_d, (int*)work_d, s), "tied build launch");
         return OTVMC_OK;
     }
     if (precision == OTVMC_PREC_FP64 && !S_d) return fail(OTVMC_ERR_INVALID, "FP64 build needs S_d");
@@ -1154,7 +1161,7 @@ static otvmc_status run_eval(const otvmc_ansatz* a, const otvmc_run_desc* d, con
     }
     if (a->kind == OTVMC_LJ) {
         CK(launch_vquant(T, ns, r.v, r.eb, s), "vquant launch");
-        CK(launch_lj_build(a, spins, T, ns, r.eb, r.obuf, r.S, r.obar, r.D, s), "tied build launch");
+        CK(launch_lj_build(a, spins, T, ns, r.eb, r.obuf, r.S, r.obar, r.D, status, s), "tied build launch");
     } else {
         st = run_build(a, spins, r.v, T, ns, d->precision, true, r.eb, r.obuf, r.S, r.G, r.obar, r.D, status, s);
         if (st) return st;
@@ -1163,8 +1170,7 @@ static otvmc_status run_eval(const otvmc_ansatz* a, const otvmc_run_desc* d, con
     if (d->reg == OTVMC_REG_SNR) {
         if (a->P > SNR_PMAX)
             CK(launch_snr_big(a, T, ns, spins, r.S, r.obar, r.v, r.D, d->snr_thresh, SNR_EPS_SVD, delta, nullptr,
-                              r.snr, status, s, d->precision == OTVMC_PREC_MIXED,
-                              a->kind == OTVMC_LJ ? lj_built_O(a, T, r.obuf) : nullptr),
+                              r.snr, status, s),
                "snr solve launch");
         else
             CK(launch_snr_solve(a, T, ns, spins, r.S, r.obar, r.v, r.D, d->snr_thresh, SNR_EPS_SVD, delta, nullptr,

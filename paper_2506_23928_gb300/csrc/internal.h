@@ -30,7 +30,7 @@ struct otvmc_ansatz {
     int m = 0;
     int64_t P = 0;
     int* pairs_d = nullptr;  // Jastrow: [P - n][2] sites (j, k), j < k
-    int2* tiles_d = nullptr; // upper-triangle tiles of the tensor-core Gram kernel
+    int2* tiles_d = nullptr; // upper-triangle tiles of the tensor-core Gram kernel (of the operand rows for OTVMC_LJ)
     int ntiles = 0;
     int rbm_t_build = 0;     // OTVMC_RBM_T_FACTORED or OTVMC_RBM_T_MATERIALISED
     // Tied Jastrow (OTVMC_LJ): the full Jastrow of the same model, on which sampling, local
@@ -38,6 +38,7 @@ struct otvmc_ansatz {
     // groups of pairs that share a parameter (pairs by their full-Jastrow pair index).
     otvmc_ansatz* full = nullptr;
     int lj_d = 0, lj_pbc = 0, ngroups = 0;
+    int nfree = 0;              // groups of the free pairs (distance <= lj_d), which come first
     int* grp_off_d = nullptr;   // [ngroups + 1]
     int* grp_pair_d = nullptr;  // [N(N-1)/2], grouped
     int* pair_grp_d = nullptr;  // [N(N-1)/2] group of each pair
@@ -261,23 +262,22 @@ inline size_t rbm_sample_bytes(const otvmc_ansatz* a, int ntraj, int ns) {
 // tied Jastrow (k_lj.cu)
 cudaError_t launch_lj_expand(const otvmc_ansatz* a, int ntraj, const double2* theta, double2* theta_full,
                              cudaStream_t s);
-// the tied log-derivatives O [ntraj][P][ns] int16 that launch_lj_build left in its workspace
-const int16_t* lj_built_O(const otvmc_ansatz* a, int ntraj, const void* ws);
 size_t lj_build_bytes(const otvmc_ansatz* a, int ntraj, int ns);
 cudaError_t launch_lj_build(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,
-                            void* ws, double* S, double* obar, double2* D, cudaStream_t s);
+                            void* ws, double* S, double* obar, double2* D, int* status, cudaStream_t s);
+// operand rows of the tensor-core build: sites, free pairs, two rows per tied distance
+int lj_operand_rows(const otvmc_ansatz* a);
 
 // SNR-filtered eigen pseudo-inverse (one CTA per trajectory, P <= SNR_PMAX)
 constexpr int SNR_PMAX = 96;
 constexpr double SNR_EPS_SVD = 1e-12;
 size_t snr_smem_bytes(int P);
-// the same filter for larger P: Householder tridiagonalisation, implicit QL, sample pass (k_snr_big.cu)
+// the same filter for larger P: Householder tridiagonalisation, implicit QL, weighted Gram matrix (k_snr_big.cu)
 size_t snr_big_ws_bytes(int ntraj, int P);
 bool snr_big_fits(int P);
 cudaError_t launch_snr_big(const otvmc_ansatz* a, int ntraj, int ns, const uint64_t* spins, const double* S,
                            const double* obar, const double2* v, const double2* D, double thr, double eps_svd,
-                           double2* delta, double* lam, void* ws, int* status, cudaStream_t s,
-                           bool fp32_pass = false, const int16_t* Oint = nullptr);
+                           double2* delta, double* lam, void* ws, int* status, cudaStream_t s);
 cudaError_t launch_snr_solve(const otvmc_ansatz* a, int ntraj, int ns, const uint64_t* spins, const double* S,
                              const double* obar, const double2* v, const double2* D, double thr, double eps_svd,
                              double2* delta, double* lam, int* status, cudaStream_t s);

@@ -5,11 +5,21 @@
 //     log psi = sum_i a_i s_i + sum_g eta_g sum_{(j,k) in g} s_j s_k,
 //     O_{a_i} = s_i,   O_{eta_g} = sum_{(j,k) in g} s_j s_k   (an integer, |O| <= group size).
 // Sampling, local estimators and observables only need the pair parameters eta_jk, so they run
-// the full-Jastrow kernels on the expanded parameters theta_full (expand kernel).  D and obar are
-// the full Jastrow's exact sums folded over each group (fold kernel).  S = G / ns - obar obar^T
-// from the integer Gram matrix G = sum_x O(x) O(x)^T, accumulated exactly in integers on the CUDA
-// cores (the tied rows reach |O| = N, so their products exceed what an FP32 tensor-core
-// accumulator holds exactly; P is N + a few N, small next to the full Jastrow's N(N+1)/2).
+// the full-Jastrow kernels on the expanded parameters theta_full (expand kernel).
+//
+// S and D come from one FP8 tensor-core Gram pass (k_gram_tc.cu), exactly.  A tied O reaches N in
+// magnitude, more than E4M3 holds and more than FP32 sums of products hold exactly; it enters as two
+// operand rows, O = 16 h + l with l in [-8, 7] and |h| <= 13 (N <= 200), so that every operand is a
+// whole number of at most 16 and every sum of products stays below 2^24 up to LJ_TC_MAX_NS samples.
+// A tied sum over all pairs at one distance D is (pairs) - 2 popcount(w xor (w shifted by D)), the
+// rotation for a ring, so that no pair list is walked.  The digits of the quantised v and a row of
+// ones ride along as in the full Jastrow's pass; S_ij = (ns G_ij - c_i c_j) / ns^2 and D are formed
+// in 64- and 128-bit integers and rounded once.
+// 100 trajectories of the 100-spin ring, P = 249, 4096 samples: 5.42 ms with the integer sums on the
+// CUDA cores (full-Jastrow D folded over the groups, 16-bit O, integer Gram), which remain for more
+// samples; 0.50 ms so (operand rows 0.28, Gram 0.09, S and D 0.10).
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace otvmc {
@@ -166,9 +176,214 @@ __global__ void S_kernel(int P, int ns, const long long* __restrict__ G, const d
     }
 }
 
+// Largest |h| is 13: 13 * 13 * ns < 2^24
+constexpr int LJ_TC_MAX_NS = 99200;
+constexpr int OB = 32;  // rows of O per batch
+
+// w, a string of 64 NW bits, shifted down (or UP) by D >= 0, zeros in
+template <int NW, bool UP>
+__device__ __forceinline__ void shift_bits(const uint64_t (&w)[NW], int D, uint64_t (&o)[NW]) {
+    const int q = D >> 6, r = D & 63;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+        uint64_t a = 0ull, b = 0ull;  // the word that lands on i, and the one whose bits come in
+#pragma unroll
+        for (int k = 0; k < NW; ++k) {
+            if (k == (UP ? i - q : i + q)) a = w[k];
+            if (k == (UP ? i - q - 1 : i + q + 1)) b = w[k];
+        }
+        if (r) o[i] = UP ? (a << r) | (b >> (64 - r)) : (a >> r) | (b << (64 - r));
+        else o[i] = a;
+    }
+}
+// E4M3 code of a whole number |d| <= 16
+__device__ __forceinline__ uint32_t e4m3_int(int d) {
+    if (d == 0) return 0u;
+    const int a = d < 0 ? -d : d, e = 31 - __clz(a);
+    return (d < 0 ? 0x80u : 0u) | ((uint32_t)(e + 7) << 3) | (uint32_t)(e <= 3 ? (a << (3 - e)) - 8 : (a >> (e - 3)) - 8);
+}
+
+// Operand rows of one trajectory: s_k (n), the free pairs (nf), then h and l of every tied distance
+// (2 nt, interleaved), then the D_XROWS extra rows (digits of q, ones); K-major, pitch bytes a row,
+// samples from ns on zero.  One thread per sample; OB rows at a time go through shared memory so
+// that the stores are 16 bytes of consecutive samples.  Bound: about 20 instructions per tied sum.
+template <int W>
+__global__ void __launch_bounds__(256) obuild8_kernel(int n, int nf, int nt, int d, int pbc, int ns, int pitch,
+                                                      const int* __restrict__ grp_pair, const int* __restrict__ pairs,
+                                                      const uint64_t* __restrict__ spins,
+                                                      const long long* __restrict__ qv, uint8_t* __restrict__ O) {
+    __shared__ __align__(16) uint8_t tile[OB][256];
+    const int t = blockIdx.y, tid = threadIdx.x, x = blockIdx.x * 256 + tid;
+    const int PO = n + nf + 2 * nt, R = PO + D_XROWS;
+    const bool live = x < ns;
+    uint64_t w[W];
+#pragma unroll
+    for (int q = 0; q < W; ++q) w[q] = live ? spins[((size_t)t * ns + x) * W + q] : 0ull;
+    // digit p of q + 8 (1 + 16 + ...) in base 16, less 8: the balanced digits
+    constexpr unsigned long long BIAS = 0x8888888888888888ull;
+    const unsigned long long q0 = live ? (unsigned long long)qv[((size_t)t * ns + x) * 2] + BIAS : BIAS;
+    const unsigned long long q1 = live ? (unsigned long long)qv[((size_t)t * ns + x) * 2 + 1] + BIAS : BIAS;
+    auto bit = [&](int j) -> uint32_t {
+        uint64_t v = w[0];
+#pragma unroll
+        for (int q = 1; q < W; ++q) v = (j >> 6) == q ? w[q] : v;
+        return (uint32_t)(v >> (j & 63)) & 1u;
+    };
+    uint8_t* Ot = O + (size_t)t * R * pitch;
+    for (int b = blockIdx.z; b * OB < R; b += gridDim.z) {
+        int val = 0;
+        for (int r = 0; r < OB; ++r) {
+            const int row = b * OB + r;  // uniform over the CTA
+            uint32_t code = 0u;
+            if (row < n) {
+                code = bit(row) ? 0x38u : 0xB8u;
+            } else if (row < n + nf) {
+                const int p = __ldg(grp_pair + row - n);
+                code = bit(__ldg(pairs + 2 * p)) == bit(__ldg(pairs + 2 * p + 1)) ? 0x38u : 0xB8u;
+            } else if (row < PO) {
+                const int g = (row - n - nf) >> 1, D = d + 1 + g;
+                const bool low = (row - n - nf) & 1;
+                if (!low || r == 0) {
+                    // pairs (j, j + D), and for a ring (j, j + D - n): disagreeing bits
+                    uint64_t u[W], v[W];
+                    shift_bits<W, false>(w, D, u);
+                    if (pbc) {
+                        shift_bits<W, true>(w, n - D, v);
+#pragma unroll
+                        for (int q = 0; q < W; ++q) u[q] |= v[q];
+                    }
+                    const int m = pbc ? n : n - D;
+                    int dis = 0;
+#pragma unroll
+                    for (int q = 0; q < W; ++q) {
+                        const int left = m - 64 * q;
+                        const uint64_t mask = left >= 64 ? ~0ull : left > 0 ? (1ull << left) - 1ull : 0ull;
+                        dis += __popcll((w[q] ^ u[q]) & mask);
+                    }
+                    // half way round an even ring every pair is met twice
+                    const bool twice = pbc && 2 * D == n;
+                    val = twice ? m / 2 - dis : m - 2 * dis;
+                }
+                const int l = ((val + 8) & 15) - 8;
+                code = e4m3_int(low ? l : (val - l) >> 4);
+            } else if (row < R) {
+                const int p = row - PO;
+                code = p == 32 ? 0x38u : e4m3_int((int)(((p < 16 ? q0 : q1) >> (4 * (p & 15))) & 15ull) - 8);
+            }
+            tile[r][tid] = live ? (uint8_t)code : (uint8_t)0;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int r = (tid >> 4) + 16 * k, row = b * OB + r, xs = blockIdx.x * 256 + 16 * (tid & 15);
+            if (row < R && xs < pitch)
+                *reinterpret_cast<uint4*>(Ot + (size_t)row * pitch + xs) =
+                    *reinterpret_cast<const uint4*>(&tile[r][16 * (tid & 15)]);
+        }
+        __syncthreads();
+    }
+}
+
+// Operand row (the h row of a tied sum) of parameter k, and whether it is tied.
+__device__ __forceinline__ int orow(int k, int nu, bool& tied) {
+    tied = k >= nu;
+    return tied ? nu + 2 * (k - nu) : k;
+}
+__device__ __forceinline__ long long count_of(const float* Xt, int row, bool tied) {
+    const long long a = (long long)Xt[(size_t)row * D_XROWS + 32];
+    return tied ? 16 * a + (long long)Xt[(size_t)(row + 1) * D_XROWS + 32] : a;
+}
+
+// obar and D from the side output of the Gram pass, X[t][row][D_XROWS]: sums over the samples of O
+// against the digits of q and the ones.
+__global__ void __launch_bounds__(128) D_kernel(int nu, int P, int PO, int ns, const float* __restrict__ X,
+                                                const double* __restrict__ vinfo, const long long* __restrict__ qsum,
+                                                double* __restrict__ obar, double2* __restrict__ D) {
+    const int t = blockIdx.y, k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= P) return;
+    const float* Xt = X + (size_t)t * PO * D_XROWS;
+    bool tied;
+    const int row = orow(k, nu, tied);
+    const long long c = count_of(Xt, row, tied);
+    double out[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        // sum_x O q, exactly (at most 200 2^60), then ns sum - c Q
+        __int128 sum = 0;
+#pragma unroll
+        for (int p = 15; p >= 0; --p) {
+            long long a = (long long)Xt[(size_t)row * D_XROWS + 16 * h + p];
+            if (tied) a = 16 * a + (long long)Xt[(size_t)(row + 1) * D_XROWS + 16 * h + p];
+            sum = sum * 16 + a;
+        }
+        const __int128 num = sum * ns - (__int128)c * qsum[2 * t + h];
+        // in two parts of 64 bits: one rounding
+        const long long hi = (long long)(num >> 53), lo = (long long)(num - ((__int128)hi << 53));
+        out[h] = fma((double)hi, 9007199254740992.0, (double)lo);
+    }
+    const double inv = vinfo[4 * t + 2] / ((double)ns * (double)ns);
+    obar[(size_t)t * P + k] = (double)c / ns;
+    D[(size_t)t * P + k] = make_double2(out[0] * inv, out[1] * inv);
+}
+
+// S (full, FP64) from the Gram counts of the operand rows (upper triangle, FP32): one 32 x 32 tile
+// of the upper triangle per CTA, mirrored through shared memory.
+__global__ void __launch_bounds__(256) S8_kernel(int nu, int P, int PO, int ns, const float* __restrict__ G,
+                                                 const float* __restrict__ X, double* __restrict__ S) {
+    constexpr int B = 32;
+    __shared__ double tile[B][B + 1];
+    __shared__ long long ci[B], cj[B];
+    const int t = blockIdx.y;
+    int J = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+    while ((J + 1) * (J + 2) / 2 <= (int)blockIdx.x) ++J;
+    while (J * (J + 1) / 2 > (int)blockIdx.x) --J;
+    const int I = blockIdx.x - J * (J + 1) / 2;
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const float* Xt = X + (size_t)t * PO * D_XROWS;
+    if (threadIdx.x < 2 * B) {
+        const int k = (threadIdx.x < B ? I : J) * B + tx;
+        bool tied;
+        const int row = orow(k, nu, tied);
+        (threadIdx.x < B ? ci : cj)[tx] = k < P ? count_of(Xt, row, tied) : 0ll;
+    }
+    __syncthreads();
+    const float* Gt = G + (size_t)t * PO * PO;
+    double* St = S + (size_t)t * P * P;
+    const double den = (double)ns * (double)ns;
+#pragma unroll
+    for (int r = ty; r < B; r += 8) {
+        const int i = I * B + r, j = J * B + tx;
+        double v = 0.0;
+        if (i < P && j < P && i <= j) {
+            bool ti, tj;
+            const int a = orow(i, nu, ti), b = orow(j, nu, tj);
+            const float* g = Gt + (size_t)a * PO + b;
+            long long s = (long long)g[0];
+            if (tj) s = 16 * s + (long long)g[1];
+            if (ti) {
+                // the l row of i against b and b + 1; on the diagonal (l, h) is (h, l)
+                const long long lo = i == j ? (long long)g[1] : (long long)g[PO];
+                s = 16 * s + (tj ? 16 * lo + (long long)g[PO + 1] : lo);
+            }
+            v = (double)(s * ns - ci[r] * cj[tx]) / den;
+            St[(size_t)i * P + j] = v;
+        }
+        tile[r][tx] = v;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = ty; r < B; r += 8) {
+        const int j = J * B + r, i = I * B + tx;
+        if (i < P && j < P && i < j) St[(size_t)j * P + i] = tile[tx][r];
+    }
+}
+
 static size_t rup(size_t b) { return (b + 255) & ~(size_t)255; }
+static int operand_rows(const otvmc_ansatz* a) { return a->n + a->nfree + 2 * (a->ngroups - a->nfree); }
 
 }  // namespace lj
+
+int lj_operand_rows(const otvmc_ansatz* a) { return lj::operand_rows(a); }
 
 cudaError_t launch_lj_expand(const otvmc_ansatz* a, int ntraj, const double2* theta, double2* theta_full,
                              cudaStream_t s) {
@@ -182,22 +397,51 @@ cudaError_t launch_lj_expand(const otvmc_ansatz* a, int ntraj, const double2* th
 
 size_t lj_build_bytes(const otvmc_ansatz* a, int ntraj, int ns) {
     using lj::rup;
-    const size_t T = (size_t)ntraj, P = (size_t)a->P, Pf = (size_t)a->full->P;
+    const size_t T = (size_t)ntraj, P = (size_t)a->P, Pf = (size_t)a->full->P, PO = (size_t)lj::operand_rows(a);
+    if (ns <= lj::LJ_TC_MAX_NS)
+        return rup(T * (PO + D_XROWS) * o_pitch(ns)) + rup(T * PO * PO * 4) + rup(T * PO * D_XROWS * 4) + 256;
     return rup(T * Pf * 8) + rup(T * Pf * 16) + rup(T * P * ns * 2) + rup(T * P * P * 8) + 256;
 }
 
-const int16_t* lj_built_O(const otvmc_ansatz* a, int ntraj, const void* ws) {
+static cudaError_t lj_build_tc(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,
+                               void* ws, double* S, double* obar, double2* D, int* status, cudaStream_t s) {
     using lj::rup;
-    const size_t T = (size_t)ntraj, Pf = (size_t)a->full->P;
-    return (const int16_t*)((const char*)ws + rup(T * Pf * 8) + rup(T * Pf * 16));
+    const int n = a->n, W = (n + 63) / 64, P = (int)a->P, nu = n + a->nfree, PO = lj::operand_rows(a);
+    const int pitch = o_pitch(ns), R = PO + D_XROWS;
+    uint8_t* O = (uint8_t*)ws;
+    float* G = (float*)((char*)ws + rup((size_t)ntraj * R * pitch));
+    float* X = (float*)((char*)G + rup((size_t)ntraj * PO * PO * 4));
+    {
+        ProfScope prof_(OTVMC_K_OBUILD, s);
+        // the row batches over gridDim.z while the batch leaves SMs without work
+        const int gx = (pitch + 255) / 256, nb = (R + lj::OB - 1) / lj::OB;
+        const int gz = std::max(1, std::min(nb, (8 * 152 + gx * ntraj - 1) / (gx * ntraj)));
+        const auto fn = W == 1 ? lj::obuild8_kernel<1> : W == 2 ? lj::obuild8_kernel<2>
+                        : W == 3 ? lj::obuild8_kernel<3> : lj::obuild8_kernel<4>;
+        fn<<<dim3(gx, ntraj, gz), 256, 0, s>>>(n, a->nfree, a->ngroups - a->nfree, a->lj_d, a->lj_pbc, ns, pitch,
+                                               a->grp_pair_d, a->full->pairs_d, spins, b.qv, O);
+        count_launch();
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+    }
+    const cudaError_t e = launch_gram_tc(ntraj, PO, R, ns, pitch, O, a->tiles_d, a->ntiles, G, X, status, s);
+    if (e != cudaSuccess) return e;
+    ProfScope prof_(OTVMC_K_D, s);
+    const int nt = (P + 31) / 32;
+    lj::D_kernel<<<dim3((P + 127) / 128, ntraj), 128, 0, s>>>(nu, P, PO, ns, X, b.vinfo, b.qsum, obar, D);
+    lj::S8_kernel<<<dim3(nt * (nt + 1) / 2, ntraj), 256, 0, s>>>(nu, P, PO, ns, G, X, S);
+    count_launch(2);
+    return cudaGetLastError();
 }
 
 // S (full FP64), obar and D of the tied parameters from the samples and the quantised v in b
-// (vpart / vquant already run on b): D and obar of the full Jastrow by the exact integer sums,
-// folded over the groups; S from the exact integer Gram matrix of the tied O.
+// (vpart / vquant already run on b).  Beyond LJ_TC_MAX_NS samples on the CUDA cores: D and obar of the
+// full Jastrow by the exact integer sums, folded over the groups; S from the exact integer Gram
+// matrix of the tied O.
 cudaError_t launch_lj_build(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,
-                            void* ws, double* S, double* obar, double2* D, cudaStream_t s) {
+                            void* ws, double* S, double* obar, double2* D, int* status, cudaStream_t s) {
     using lj::rup;
+    if (ns <= lj::LJ_TC_MAX_NS) return lj_build_tc(a, spins, ntraj, ns, b, ws, S, obar, D, status, s);
     const otvmc_ansatz* f = a->full;
     const int n = a->n, P = (int)a->P, Pf = (int)f->P, W = (n + 63) / 64;
     char* q = (char*)ws;

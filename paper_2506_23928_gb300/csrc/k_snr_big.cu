@@ -4,29 +4,37 @@
 //     SNR_k = |rho_k| / sqrt(Var_x Q_k / ns),
 //     f_k = 1 / (1 + (thr / SNR_k)^6) * 1 / (1 + (eps_svd lambda_max / lambda_k)^6),
 //     delta = V diag(f_k / lambda_k) rho   (lambda_k <= 0 dropped),
-// with the eigen-decomposition done by
-//   (1) Householder tridiagonalisation of a copy A of S: T = Q^T A Q, Q = H_0 H_1 ... H_{P-3},
-//       H_k = I - tau_k v_k v_k^T acting on indices k+1 .. P-1 (v_k kept in column k of A);
-//   (2) Q^T formed explicitly, as X = H_{P-3}, then X <- X H_k for k = P-4 .. 0, each step
-//       touching only the trailing block that H_k acts on;
-//   (3) the implicit QL iteration with the shift from the leading 2 x 2 block on T (d, e),
-//       every plane rotation applied to the rows of X, so that at the end row k of X is the
-//       eigenvector of eigenvalue d_k (X = V^T); eigenvalues to an absolute accuracy of a few
-//       eps ||S||, as a dense symmetric eigensolver gives them;
-// then (4) rho and one pass over the samples for the mean and the second moment of Q_k, and
-// (5) the filter and the back-projection.  One CTA per trajectory, FP64 throughout; A and X
-// live in the caller's workspace (2 P^2 doubles per trajectory), d, e, the reflector and the
-// rotations of a QL sweep in shared memory.  The scalar recurrence of a QL sweep runs on one
-// thread; the sweep's rotations are then applied to all columns of X at once.
+// in five launches, all in FP64 or exact integers:
+//   tri    Householder tridiagonalisation of a copy A of S: T = Q^T A Q, Q = H_0 H_1 ... H_{P-3},
+//          H_k = I - tau_k v_k v_k^T acting on indices k+1 .. P-1 (v_k kept in column k of A); then
+//          Q^T explicitly, as X = H_{P-3}, X <- X H_k for k = P-4 .. 0, each step touching only the
+//          trailing block that H_k acts on.  One CTA per trajectory.
+//   wgram  M = sum_x w(x) O_c(x) O_c(x)^T, w = |v_c|^2, into A's place: Var_x Q_k = v_k^T M v_k / ns -
+//          |rho_k|^2, which takes P^2 products per sample once for all k, half of them by symmetry,
+//          in place of the P^2 FP64 products of the projections y_k(x).  w as a 46-bit integer in two
+//          digits of 23 bits, O as the small integer that it is: every product and sum is exact in
+//          64-bit integers, which run at 16 times the FP64 rate.  One CTA per 64 x 64 tile.
+//   ql     the implicit QL iteration with the shift from the leading 2 x 2 block on T (d, e), every
+//          plane rotation applied to the rows of X, so that at the end row k of X is the eigenvector
+//          of eigenvalue d_k (X = V^T); eigenvalues to an absolute accuracy of a few eps ||S||, as a
+//          dense symmetric eigensolver gives them.  One CTA per trajectory: one warp runs the scalar
+//          recurrence of a sweep while eight apply the rotations of the sweep before.
+//   var    v_k^T M v_k, an FP64 product per 32 eigenvectors.
+//   final  rho, the filter and the back-projection.
+// Bound: FP64 at 2 multiply-adds per cycle and SM (tri: about 5/3 P^3 of them, ql: 2 per rotation and
+// column, about 3 P^3, var: P^3), and in ql the chain of the recurrence (about 0.85 P^2 rotations).
+// 100 trajectories of P = 249, 4096 samples, in one kernel with FP64 projections of every sample
+// and the recurrence between the rotations: 321 ms; now 85 ms (tri 18, wgram 10, ql 53, var 3).
+// A and X live in the caller's workspace (2 P^2 doubles per trajectory).  Only the upper triangle of M
+// is stored; d, e and v^T M v pass from launch to launch in the lower one (SnrScratch).
 #include "common.cuh"
 
 namespace otvmc {
 
-constexpr int SNRB_THREADS = 256;
+constexpr int SNRB_THREADS = 512;
 constexpr int SNRB_WARPS = SNRB_THREADS / 32;
 constexpr int SNRB_MAX_ITER = 60;        // QL iterations per eigenvalue before giving up
-constexpr int SNRB_SMEM_BUDGET = 216 * 1024;  // + the signs of a chunk of samples
-constexpr int SNRB_SGN_BYTES = 16 * 200;          // 16 samples x N <= 200 sites
+constexpr int SNRB_SMEM_BUDGET = 216 * 1024;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
@@ -34,7 +42,8 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Sum over the CTA (every thread calls it; red holds SNRB_WARPS doubles).
+// Sum over a CTA of NW warps (every thread calls it; red holds NW doubles).
+template <int NW>
 __device__ double block_sum(double v, double* red) {
     v = warp_sum(v);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -43,117 +52,32 @@ __device__ double block_sum(double v, double* red) {
     __syncthreads();
     double s = 0.0;
 #pragma unroll
-    for (int i = 0; i < SNRB_WARPS; ++i) s += red[i];
+    for (int i = 0; i < NW; ++i) s += red[i];
     return s;
 }
 
-// Samples per chunk of the sample pass, chosen so that the shared memory fits the budget.
-__host__ __device__ inline int snrb_chunk(int P) {
-    const int c = (SNRB_SMEM_BUDGET / 8 - 7 * P - 33) / P;
-    return c > 16 ? 16 : c;
-}
-
-template <typename T>
-__device__ __forceinline__ T warp_sum_t(T v) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    return v;
-}
-
-// One pass over the samples in chunks of CH held in shared memory (och): per eigenvector k
-// (row k of V), the sums over x of Q_k(x) = y_k(x) v_c(x), y_k(x) = sum_i V_ki O_c,i(x), and of
-// |Q_k(x)|^2, added to qs[k] and q2[k].  One warp per k; y in T, Q and the sums in FP64.
-template <typename T>
-__device__ void snrb_sample_pass(int n, int W, int P, int ns, const uint64_t* sp, const int* pairs,
-                                 const int* grp_off, const int* grp_pair, const int16_t* Oint, const double* ob,
-                                 const T* V, T* och, signed char* sgn, int CH, const double2* vt, double vbx,
-                                 double vby, double2* qs, double* q2) {
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    for (int x0 = 0; x0 < ns; x0 += CH) {
-        const int nc = min(CH, ns - x0);
-        if (Oint != nullptr) {
-            // the log-derivatives already built as integers ([P][ns] of this trajectory)
-            for (int q = tid; q < nc * P; q += blockDim.x) {
-                const int i = q / nc, c = q % nc;
-                och[(size_t)c * P + i] = (T)((double)Oint[(size_t)i * ns + x0 + c] - ob[i]);
-            }
-        } else {
-            // the chunk's spins as signs in shared memory, then O - obar from them
-            for (int q = tid; q < nc * n; q += blockDim.x) {
-                const int c = q / n, j = q % n;
-                sgn[c * n + j] = (signed char)spin_of(sp + (size_t)(x0 + c) * W, j);
-            }
-            __syncthreads();
-            for (int q = tid; q < nc * P; q += blockDim.x) {
-                const int c = q / P, i = q % P;
-                const signed char* sg = sgn + c * n;
-                int o;
-                if (i < n) {
-                    o = sg[i];
-                } else if (grp_off == nullptr) {
-                    o = sg[pairs[2 * (i - n)]] * sg[pairs[2 * (i - n) + 1]];
-                } else {
-                    o = 0;
-                    for (int e = grp_off[i - n]; e < grp_off[i - n + 1]; ++e) {
-                        const int pp = grp_pair[e];
-                        o += sg[pairs[2 * pp]] * sg[pairs[2 * pp + 1]];
-                    }
-                }
-                och[(size_t)c * P + i] = (T)((double)o - ob[i]);
-            }
-        }
-        __syncthreads();
-        for (int k = warp; k < P; k += SNRB_WARPS) {
-            const T* Vk = V + (size_t)k * P;
-            T y[16];
-#pragma unroll
-            for (int c = 0; c < 16; ++c) y[c] = (T)0;
-            for (int i = lane; i < P; i += 32) {
-                const T vk = Vk[i];
-#pragma unroll
-                for (int c = 0; c < 16; ++c)
-                    if (c < nc) y[c] += vk * och[(size_t)c * P + i];
-            }
-            double ax = 0.0, ay = 0.0, a2 = 0.0;
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                if (c >= nc) break;
-                const double yc = (double)warp_sum_t(y[c]);
-                const double vx = vt[x0 + c].x - vbx, vy = vt[x0 + c].y - vby;
-                const double qx = yc * vx, qy = yc * vy;
-                ax += qx;
-                ay += qy;
-                a2 += qx * qx + qy * qy;
-            }
-            if (lane == 0) {
-                qs[k].x += ax;
-                qs[k].y += ay;
-                q2[k] += a2;
-            }
-        }
-        __syncthreads();
+// d_k (then the eigenvalue) and e_k (then v_k^T M v_k) in the strict lower triangle of A, once the
+// reflectors there are no longer needed: rows P - 1 and P - 2, what does not fit in row P - 3.
+struct SnrScratch {
+    double* A;
+    int P;
+    __device__ double& d(int k) const { return k < P - 1 ? A[(size_t)(P - 1) * P + k] : A[(size_t)(P - 3) * P]; }
+    __device__ double& e(int k) const {
+        return k < P - 2 ? A[(size_t)(P - 2) * P + k] : A[(size_t)(P - 3) * P + 1 + (k - (P - 2))];
     }
-}
+};
 
-__global__ void __launch_bounds__(SNRB_THREADS, 1) snr_big_kernel(
-    int n, int W, int P, int ns, const uint64_t* __restrict__ spins, const int* __restrict__ pairs,
-    const int* __restrict__ grp_off, const int* __restrict__ grp_pair, const double* __restrict__ S,
-    const double* __restrict__ obar, const double2* __restrict__ v, const double2* __restrict__ D, double thr,
-    double eps_svd, double* __restrict__ Aws, double* __restrict__ Xws, double2* __restrict__ delta,
-    double* __restrict__ lam_out, int* status, int fp32_pass, const int16_t* __restrict__ Oint) {
+// ------------------------------------------------------------------- tridiagonalisation
+__global__ void __launch_bounds__(SNRB_THREADS, 1) snr_tri_kernel(int P, const double* __restrict__ S,
+                                                                  double* __restrict__ Aws, double* __restrict__ Xws) {
     const int t = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     extern __shared__ __align__(16) double sm[];
-    double* d = sm;            // [P] diagonal, then the eigenvalues
+    double* d = sm;            // [P] diagonal
     double* e = d + P;         // [P] subdiagonal (e[i] couples i and i + 1)
     double* tau = e + P;       // [P]
     double* vb = tau + P;      // [P] reflector
     double* pb = vb + P;       // [P] p, then w
-    double* cs = pb + P;       // [P] rotation cosines of a QL sweep
-    double* ss = cs + P;       // [P] rotation sines
-    double* red = ss + P;      // [32] (+1 for odd P: och stays 16-byte aligned)
-    double* och = red + 32 + (P & 1);  // [CH][P] centred O of a chunk of samples
-    signed char* sgn = reinterpret_cast<signed char*>(och + (size_t)snrb_chunk(P) * P);  // [CH][N] spins
-    __shared__ int ql_l, ql_m, ql_lo, ql_done, ql_fail;
+    double* red = pb + P;      // [SNRB_WARPS]
     const size_t PP = (size_t)P * P;
     double* A = Aws + (size_t)t * PP;
     double* X = Xws + (size_t)t * PP;
@@ -161,7 +85,6 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_big_kernel(
     for (size_t i = tid; i < PP; i += blockDim.x) A[i] = St[i];
     __syncthreads();
 
-    // ---- (1) tridiagonalisation
     for (int k = 0; k + 2 < P; ++k) {
         const int m = P - 1 - k;
         double s2 = 0.0;
@@ -170,7 +93,7 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_big_kernel(
             vb[i] = x;
             s2 += x * x;
         }
-        const double nrm2 = block_sum(s2, red);
+        const double nrm2 = block_sum<SNRB_WARPS>(s2, red);
         const double x0 = vb[0];
         const double alpha = nrm2 > 0.0 ? -copysign(sqrt(nrm2), x0) : 0.0;
         const double vtv = nrm2 - 2.0 * alpha * x0 + alpha * alpha;
@@ -188,6 +111,7 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_big_kernel(
             for (int i = warp; i < m; i += SNRB_WARPS) {
                 const double* Bi = A + (size_t)(k + 1 + i) * P + k + 1;
                 double s = 0.0;
+#pragma unroll 8
                 for (int j = lane; j < m; j += 32) s += Bi[j] * vb[j];
                 s = warp_sum(s);
                 if (lane == 0) pb[i] = tk * s;
@@ -195,13 +119,14 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_big_kernel(
             __syncthreads();
             double pv = 0.0;
             for (int i = tid; i < m; i += blockDim.x) pv += pb[i] * vb[i];
-            const double K = 0.5 * tk * block_sum(pv, red);
+            const double K = 0.5 * tk * block_sum<SNRB_WARPS>(pv, red);
             for (int i = tid; i < m; i += blockDim.x) pb[i] -= K * vb[i];  // w = p - K v
             __syncthreads();
             // B -= v w^T + w v^T
             for (int i = warp; i < m; i += SNRB_WARPS) {
                 double* Bi = A + (size_t)(k + 1 + i) * P + k + 1;
                 const double vi = vb[i], wi = pb[i];
+#pragma unroll 8
                 for (int j = lane; j < m; j += 32) Bi[j] -= vi * pb[j] + wi * vb[j];
             }
         }
@@ -213,15 +138,13 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_big_kernel(
         if (P >= 2) {
             d[P - 2] = A[(size_t)(P - 2) * P + P - 2];
             e[P - 2] = A[(size_t)(P - 1) * P + P - 2];
-            tau[P - 2] = 0.0;
         }
         d[P - 1] = A[(size_t)(P - 1) * P + P - 1];
         e[P - 1] = 0.0;
-        tau[P - 1] = 0.0;
     }
     __syncthreads();
 
-    // ---- (2) X = Q^T = H_{P-3} ... H_0, formed as X <- X H_k from the identity, k descending
+    // X = Q^T = H_{P-3} ... H_0, formed as X <- X H_k from the identity, k descending
     for (size_t i = tid; i < PP; i += blockDim.x) X[i] = (i / P == i % P) ? 1.0 : 0.0;
     __syncthreads();
     for (int k = P - 3; k >= 0; --k) {
@@ -231,88 +154,321 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_big_kernel(
         for (int i = tid; i < m; i += blockDim.x) vb[i] = A[(size_t)(k + 1 + i) * P + k];
         __syncthreads();
         // rows r >= k + 1 of X are the only ones with entries in columns k + 1 .. (X is the
-        // identity elsewhere): u_r = (X v)_r, then X[r][k+1+b] -= tau u_r v_b
-        for (int r = warp; r < m; r += SNRB_WARPS) {
-            const double* Xr = X + (size_t)(k + 1 + r) * P + k + 1;
-            double s = 0.0;
-            for (int b = lane; b < m; b += 32) s += Xr[b] * vb[b];
-            s = warp_sum(s);
-            if (lane == 0) pb[r] = tk * s;
-        }
-        __syncthreads();
+        // identity elsewhere): u_r = (X v)_r, then X[r][k+1+b] -= tau u_r v_b, a warp per row
         for (int r = warp; r < m; r += SNRB_WARPS) {
             double* Xr = X + (size_t)(k + 1 + r) * P + k + 1;
-            const double u = pb[r];
+            double s = 0.0;
+#pragma unroll 8
+            for (int b = lane; b < m; b += 32) s += Xr[b] * vb[b];
+            const double u = tk * warp_sum(s);
+#pragma unroll 8
             for (int b = lane; b < m; b += 32) Xr[b] -= u * vb[b];
         }
         __syncthreads();
     }
+    const SnrScratch sc{A, P};
+    for (int i = tid; i < P; i += blockDim.x) {
+        sc.d(i) = d[i];
+        sc.e(i) = e[i];
+    }
+}
 
-    // ---- (3) implicit QL on (d, e); rotations applied to rows i, i + 1 of X
-    if (tid == 0) {
-        ql_l = 0;
-        ql_done = 0;
-        ql_fail = 0;
+// ------------------------------------------------------------------------- weighted Gram
+constexpr int WG = 64;   // tile
+constexpr int WK = 32;   // samples per chunk
+constexpr int WBITS = 23;
+
+// O_k of a sample with spin words w[W] (shared memory): s_k, s_j s_l, or the sum over a tied group.
+struct OShape {
+    int n, W, P, nu;      // nu: parameters that are single spins or pairs
+    int d, pbc;           // tied distances d + 1 + (k - nu)
+    const int* pairs;     // pairs of the full Jastrow
+    const int* grp_pair;  // tied ansatz: the free groups' pairs (nullptr: parameter n + q is pair q)
+};
+__device__ __forceinline__ int o_value(const OShape& o, const uint64_t* w, int k) {
+    if (k < o.n) return spin_of(w, k);
+    if (k < o.nu) {
+        const int p = o.grp_pair ? __ldg(o.grp_pair + k - o.n) : k - o.n;
+        const int2 jl = __ldg(reinterpret_cast<const int2*>(o.pairs) + p);
+        return spin_of(w, jl.x) * spin_of(w, jl.y);
+    }
+    // all pairs at distance D: (pairs) - 2 (disagreeing ones), from the string shifted by D (rotated
+    // for a ring, where each pair half way round is met twice)
+    const int D = o.d + 1 + k - o.nu, m = o.pbc ? o.n : o.n - D;
+    int dis = 0;
+    for (int q = 0; q < o.W; ++q) {
+        const int left = m - 64 * q;
+        if (left <= 0) break;
+        uint64_t u = 0ull;
+        {
+            const int b = 64 * q + D, i = b >> 6, r = b & 63;
+            if (i < o.W) u = w[i] >> r;
+            if (r && i + 1 < o.W) u |= w[i + 1] << (64 - r);
+        }
+        if (o.pbc) {  // bits n - D and up take the string's first bits
+            const int b = 64 * q - (o.n - D), i = b >> 6, r = b & 63;  // (arithmetic shift: b may be negative)
+            if (i >= 0 && i < o.W) u |= w[i] >> r;
+            if (i + 1 >= 0 && i + 1 < o.W && r) u |= w[i + 1] << (64 - r);
+        }
+        const uint64_t mask = left >= 64 ? ~0ull : (1ull << left) - 1ull;
+        dis += __popcll((w[q] ^ u) & mask);
+    }
+    return o.pbc && 2 * D == o.n ? m / 2 - dis : m - 2 * dis;
+}
+
+__device__ __forceinline__ double to_double(__int128 v) {
+    const long long hi = (long long)(v >> 53), lo = (long long)(v - ((__int128)hi << 53));
+    // (hi may take more than 53 bits: then its conversion is the one rounding that counts)
+    return fma((double)hi, 9007199254740992.0, (double)lo);
+}
+
+// The upper triangle of M, a 64 x 64 tile per CTA.
+__global__ void __launch_bounds__(256) snr_wgram_kernel(OShape o, int ns, const uint64_t* __restrict__ spins,
+                                                        const double2* __restrict__ v,
+                                                        const double* __restrict__ obar, double* __restrict__ M) {
+    const int t = blockIdx.y, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    int J = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
+    while ((J + 1) * (J + 2) / 2 <= (int)blockIdx.x) ++J;
+    while (J * (J + 1) / 2 > (int)blockIdx.x) --J;
+    const int I = blockIdx.x - J * (J + 1) / 2, r0 = I * WG, c0 = J * WG, P = o.P, W = o.W;
+    __shared__ __align__(16) int As[WK][WG];           // O of the tile's rows
+    __shared__ __align__(16) int B1[WK][WG], B0[WK][WG];  // O of its columns times the digits of w
+    __shared__ uint64_t sw[WK][4];
+    __shared__ int q1s[WK], q0s[WK];
+    __shared__ double red[8];
+    __shared__ long long redl[16];
+    __shared__ long long mrow[2 * WG][2];              // sums of w O, digit sums, rows then columns
+    const double2* vt = v + (size_t)t * ns;
+    const uint64_t* sp = spins + (size_t)t * ns * W;
+    // mean of v, largest w
+    double sx = 0.0, sy = 0.0;
+    for (int x = tid; x < ns; x += 256) {
+        sx += vt[x].x;
+        sy += vt[x].y;
+    }
+    const double vbx = block_sum<8>(sx, red) / ns, vby = block_sum<8>(sy, red) / ns;
+    double wm = 0.0;
+    for (int x = tid; x < ns; x += 256) {
+        const double a = vt[x].x - vbx, b = vt[x].y - vby;
+        wm = fmax(wm, a * a + b * b);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) wm = fmax(wm, __shfl_xor_sync(0xffffffffu, wm, off));
+    __syncthreads();
+    if ((tid & 31) == 0) red[tid >> 5] = wm;
+    __syncthreads();
+    wm = red[0];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) wm = fmax(wm, red[i]);
+    int ex = 0;
+    if (wm > 0.0 && wm < 1e300) frexp(wm, &ex);  // wm < 2^ex
+    const int sh = 2 * WBITS - ex;
+    const double up = ldexp(1.0, sh < 1000 ? sh : 1000);
+
+    long long a1[4][4], a0[4][4], ws1 = 0, ws0 = 0, m1 = 0, m0 = 0;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) a1[a][b] = a0[a][b] = 0;
+    for (int x0 = 0; x0 < ns; x0 += WK) {
+        __syncthreads();
+        for (int e = tid; e < WK * W; e += 256) {
+            const int x = e / W, q = e - x * W;
+            sw[x][q] = x0 + x < ns ? sp[(size_t)(x0 + x) * W + q] : 0ull;
+        }
+        if (tid < WK) {
+            long long q = 0;
+            if (x0 + tid < ns) {
+                const double a = vt[x0 + tid].x - vbx, b = vt[x0 + tid].y - vby;
+                q = __double2ll_rn((a * a + b * b) * up);
+            }
+            const long long top = (1ll << (2 * WBITS)) - 1;  // a w just below 2^ex may round up to it
+            q = q < 0 ? 0 : q > top ? top : q;
+            q1s[tid] = (int)(q >> WBITS);
+            q0s[tid] = (int)(q & ((1ll << WBITS) - 1));
+        }
+        __syncthreads();
+        for (int e = tid; e < 2 * WK * WG; e += 256) {
+            const int x = (e >> 6) & (WK - 1), r = e & (WG - 1);
+            const bool col = e >= WK * WG;  // uniform over a warp
+            const int k = (col ? c0 : r0) + r;
+            const int val = k < P ? o_value(o, sw[x], k) : 0;
+            if (col) {
+                B1[x][r] = val * q1s[x];
+                B0[x][r] = val * q0s[x];
+            } else {
+                As[x][r] = val;
+            }
+        }
+        __syncthreads();
+        if (tid < WG) {  // sums of w O of the rows, then of the columns; of w by one thread
+#pragma unroll 4
+            for (int x = 0; x < WK; ++x) {
+                m1 += (long long)As[x][tid] * q1s[x];
+                m0 += (long long)As[x][tid] * q0s[x];
+            }
+        } else if (tid < 2 * WG) {
+#pragma unroll 4
+            for (int x = 0; x < WK; ++x) {
+                m1 += B1[x][tid - WG];
+                m0 += B0[x][tid - WG];
+            }
+        } else if (tid == 2 * WG) {
+            for (int x = 0; x < WK; ++x) {
+                ws1 += q1s[x];
+                ws0 += q0s[x];
+            }
+        }
+#pragma unroll 4
+        for (int x = 0; x < WK; ++x) {
+            const int4 av = *reinterpret_cast<const int4*>(&As[x][4 * ty]);
+            const int4 b1 = *reinterpret_cast<const int4*>(&B1[x][4 * tx]), b0 = *reinterpret_cast<const int4*>(&B0[x][4 * tx]);
+            const int ar[4] = {av.x, av.y, av.z, av.w}, u1[4] = {b1.x, b1.y, b1.z, b1.w}, u0[4] = {b0.x, b0.y, b0.z, b0.w};
+#pragma unroll
+            for (int a = 0; a < 4; ++a)
+#pragma unroll
+                for (int b = 0; b < 4; ++b) {
+                    a1[a][b] += (long long)ar[a] * u1[b];
+                    a0[a][b] += (long long)ar[a] * u0[b];
+                }
+        }
+    }
+    if (tid < 2 * WG) {
+        mrow[tid][0] = m1;
+        mrow[tid][1] = m0;
+    } else if (tid == 2 * WG) {
+        redl[0] = ws1;
+        redl[1] = ws0;
     }
     __syncthreads();
-    int iter = 0;
+    // centred: sum w (O_i - obar_i)(O_j - obar_j), exactly through c = ns obar where that is whole (the
+    // column means of the samples), else in FP64
+    const __int128 Wt = ((__int128)redl[0] << WBITS) + redl[1];
+    const double down = ldexp(1.0, sh < 1000 ? -sh : -1000);
+    const double* ob = obar + (size_t)t * P;
+    double* Mt = M + (size_t)t * P * P;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            const int i = r0 + 4 * ty + a, j = c0 + 4 * tx + b;
+            if (i >= P || j >= P || i > j) continue;
+            const __int128 Mij = ((__int128)a1[a][b] << WBITS) + a0[a][b];
+            const __int128 mi = ((__int128)mrow[4 * ty + a][0] << WBITS) + mrow[4 * ty + a][1];
+            const __int128 mj = ((__int128)mrow[WG + 4 * tx + b][0] << WBITS) + mrow[WG + 4 * tx + b][1];
+            const double oi = ob[i], oj = ob[j];
+            const long long ci = __double2ll_rn(oi * ns), cj = __double2ll_rn(oj * ns);
+            double val;
+            if (fabs(oi * ns - (double)ci) < 1e-3 && fabs(oj * ns - (double)cj) < 1e-3) {
+                const __int128 num = (Mij * ns - (mj * ci + mi * cj)) * ns + Wt * ci * cj;
+                val = to_double(num) / ((double)ns * (double)ns) * down;
+            } else {
+                val = (to_double(Mij) - oi * to_double(mj) - oj * (to_double(mi) - oi * to_double(Wt))) * down;
+            }
+            Mt[(size_t)i * P + j] = val;
+        }
+}
+
+// --------------------------------------------------------------------------- QL iteration
+constexpr int QL_APPLY = 256;  // threads that apply rotations, a column of X each
+
+__global__ void __launch_bounds__(32 + QL_APPLY, 1) snr_ql_kernel(int P, double* __restrict__ Aws,
+                                                                  double* __restrict__ Xws, int* status) {
+    const int t = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    extern __shared__ __align__(16) double sm[];
+    double* d = sm;          // [P] diagonal, becoming the eigenvalues
+    double* e = d + P;       // [P] subdiagonal
+    double* cs2 = e + P;     // [2][P] rotations of two sweeps
+    double* ss2 = cs2 + 2 * P;
+    __shared__ int sm_m[2], sm_lo[2], sm_done[2], sm_fail;
+    double* X = Xws + (size_t)t * P * P;
+    const SnrScratch sc{Aws + (size_t)t * P * P, P};
+    for (int i = tid; i < P; i += blockDim.x) {
+        d[i] = sc.d(i);
+        e[i] = sc.e(i);
+    }
+    if (tid == 0) sm_fail = 0;
+    __syncthreads();
     // deflation: |e_m| below eps of the neighbouring diagonal entries, or below eps of the norm of
     // T (the accuracy the decomposition has anyway; without it a block of eigenvalues at the
     // rounding level of a rank-deficient S, where e stays at that level, never deflates)
+    constexpr double EPS = 2.220446049250313e-16;
     double tol_abs = 0.0;
-    if (tid == 0) {
+    int l = 0, iter = 0;
+    if (warp == 0) {
         double tn = 0.0;
-        for (int i = 0; i < P; ++i) tn = fmax(tn, fabs(d[i]) + fabs(e[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0));
-        tol_abs = 2.220446049250313e-16 * tn;
+        for (int i = lane; i < P; i += 32) tn = fmax(tn, fabs(d[i]) + fabs(e[i]) + (i > 0 ? fabs(e[i - 1]) : 0.0));
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) tn = fmax(tn, __shfl_xor_sync(0xffffffffu, tn, off));
+        tol_abs = EPS * tn;
     }
-    while (true) {
-        if (tid == 0) {
-            // find the next unreduced block starting at l; run one QL sweep on it
-            int l = ql_l, m = l, lo = -1;
-            bool swept = false;
-            while (l < P && !swept) {
-                for (m = l; m < P - 1; ++m) {
-                    const double dd = fabs(d[m]) + fabs(d[m + 1]);
-                    if (fabs(e[m]) <= tol_abs || fabs(e[m]) <= 2.220446049250313e-16 * dd) break;
-                }
-                if (m == l) {  // d[l] converged
-                    ++l;
-                    iter = 0;
-                    continue;
-                }
-                if (++iter > SNRB_MAX_ITER) {
-                    ql_fail = 1;
-                    l = P;
+    for (int step = 0;; ++step) {
+        if (warp == 0) {
+            // the next unreduced block from l on, found by the warp; then one QL sweep by its lane 0
+            const int buf = step & 1;
+            double *cs = cs2 + buf * P, *ss = ss2 + buf * P;
+            int m = l, done = 0, fail = 0;
+            while (true) {
+                if (l >= P) {
+                    done = 1;
                     break;
                 }
+                for (m = l;; m += 32) {
+                    const int i = m + lane;
+                    bool small = i >= P - 1;
+                    if (i < P - 1) small = fabs(e[i]) <= tol_abs || fabs(e[i]) <= EPS * (fabs(d[i]) + fabs(d[i + 1]));
+                    const unsigned hit = __ballot_sync(0xffffffffu, small);
+                    if (hit) {
+                        m += __ffs((int)hit) - 1;
+                        break;
+                    }
+                }
+                if (m > l) break;
+                ++l;  // d[l] converged
+                iter = 0;
+            }
+            if (!done && ++iter > SNRB_MAX_ITER) done = fail = 1;
+            int lo = m;
+            if (!done && lane == 0) {
                 double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
                 double r = hypot(g, 1.0);
                 g = d[m] - d[l] + e[l] / (g + copysign(r, g));
                 double s = 1.0, c = 1.0, p = 0.0;
-                int i = m - 1;
+                double ei = e[m - 1], di = d[m - 1], dn = d[m];  // e[i], d[i], d[i + 1]
                 bool underflow = false;
+                int i = m - 1;
                 for (; i >= l; --i) {
-                    double f = s * e[i];
-                    const double b = c * e[i];
-                    r = sqrt(f * f + g * g);
-                    if (!(r > 1e-150)) r = hypot(f, g);  // squares below the normal range
+                    const int ip = i > l ? i - 1 : l;
+                    const double en = e[ip], dp = d[ip];  // ahead of the stores below
+                    const double f = s * ei, b = c * ei;
+                    const double h2 = fma(f, f, g * g);
+                    double ir;
+                    if (h2 > 1e-290) {
+                        ir = rsqrt(h2);
+                        r = h2 * ir;
+                    } else {  // squares below the normal range
+                        r = hypot(f, g);
+                        ir = r > 0.0 ? 1.0 / r : 0.0;
+                    }
                     e[i + 1] = r;
                     if (r == 0.0) {  // deflation inside the sweep
-                        d[i + 1] -= p;
+                        d[i + 1] = dn - p;
                         e[m] = 0.0;
                         underflow = true;
                         break;
                     }
-                    const double ir = 1.0 / r;
                     s = f * ir;
                     c = g * ir;
-                    g = d[i + 1] - p;
-                    r = (d[i] - g) * s + 2.0 * c * b;
+                    g = dn - p;
+                    r = fma(di - g, s, 2.0 * c * b);
                     p = s * r;
                     d[i + 1] = g + p;
-                    g = c * r - b;
+                    g = fma(c, r, -b);
                     cs[i] = c;
                     ss[i] = s;
+                    ei = en;
+                    dn = di;
+                    di = dp;
                 }
                 lo = i + 1;  // rotations recorded for i = m - 1 .. lo
                 if (!underflow) {
@@ -320,157 +476,194 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_big_kernel(
                     e[l] = g;
                     e[m] = 0.0;
                 }
-                swept = true;
             }
-            ql_l = l;
-            ql_m = m;
-            ql_lo = lo;
-            ql_done = (l >= P) ? 1 : 0;
-        }
-        __syncthreads();
-        if (ql_done) break;
-        // apply rotations i = m - 1 down to lo to every column of X: rows i and i + 1
-        {
-            const int m = ql_m, lo = ql_lo;
-            for (int col = tid; col < P; col += blockDim.x) {
-                if (m - 1 < lo) break;
-                double zi1 = X[(size_t)m * P + col];  // row i + 1 for i = m - 1
-                // rows are loaded eight at a time ahead of the rotations that use them (each
-                // row is stored only after it has been loaded)
-                for (int i = m - 1; i >= lo; i -= 8) {
-                    const int nb = min(8, i - lo + 1);
-                    double z[8];
+            if (lane == 0) {
+                sm_m[buf] = m;
+                sm_lo[buf] = lo;
+                sm_done[buf] = done;
+                if (fail) sm_fail = 1;
+            }
+            __syncwarp();
+        } else if (step > 0) {
+            // rotations i = m - 1 down to lo of the sweep before, on rows i and i + 1 of every column
+            const int buf = (step - 1) & 1, m = sm_m[buf], lo = sm_lo[buf];
+            const double *cs = cs2 + buf * P, *ss = ss2 + buf * P;
+            if (m - 1 >= lo)
+                for (int col = tid - 32; col < P; col += QL_APPLY) {
+                    double zi1 = X[(size_t)m * P + col];  // row i + 1 for i = m - 1
+                    // rows are loaded ahead of the rotations that use them (each row is stored only
+                    // after it has been loaded)
+                    constexpr int U = 16;
+                    for (int i = m - 1; i >= lo; i -= U) {
+                        const int nb = min(U, i - lo + 1);
+                        double z[U];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (u < nb) z[u] = X[(size_t)(i - u) * P + col];
+                        for (int u = 0; u < U; ++u)
+                            if (u < nb) z[u] = X[(size_t)(i - u) * P + col];
 #pragma unroll
-                    for (int u = 0; u < 8; ++u)
-                        if (u < nb) {
-                            const double c = cs[i - u], s = ss[i - u];
-                            X[(size_t)(i - u + 1) * P + col] = s * z[u] + c * zi1;
-                            zi1 = c * z[u] - s * zi1;
-                        }
+                        for (int u = 0; u < U; ++u)
+                            if (u < nb) {
+                                const double c = cs[i - u], s = ss[i - u];
+                                X[(size_t)(i - u + 1) * P + col] = fma(s, z[u], c * zi1);
+                                zi1 = fma(c, z[u], -s * zi1);
+                            }
+                    }
+                    X[(size_t)lo * P + col] = zi1;
                 }
-                X[(size_t)lo * P + col] = zi1;
-            }
         }
+        // (the step that finds nothing left to do still applies the sweep before it; its flag is not
+        // written again before the barrier of the next step but one)
         __syncthreads();
+        if (sm_done[step & 1]) break;
     }
-    if (ql_fail) {
-        if (tid == 0) record_error(status, OTVMC_ERR_NONFINITE, t);
-        for (int i = tid; i < P; i += blockDim.x) delta[(size_t)t * P + i] = make_double2(0.0, 0.0);
+    if (sm_fail && tid == 0) record_error(status, OTVMC_ERR_NONFINITE, t);
+    // eigenvalues; NaN marks a decomposition that did not converge
+    for (int i = tid; i < P; i += blockDim.x) sc.d(i) = sm_fail ? NAN : d[i];
+}
+
+// ------------------------------------------------------------------------------- variances
+// q2_k = v_k^T M v_k of 32 eigenvectors (rows of X) per CTA, in e's place.
+__global__ void __launch_bounds__(256) snr_var_kernel(int P, const double* __restrict__ Xws, double* Mws) {
+    constexpr int BR = 32, BJ = 64, BI = 16;
+    __shared__ double As[BI][BR + 1], Bs[BI][BJ];
+    const int t = blockIdx.y, k0 = blockIdx.x * BR, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const double* X = Xws + (size_t)t * P * P;
+    double* M = Mws + (size_t)t * P * P;
+    double q2[2] = {0.0, 0.0};
+    for (int j0 = 0; j0 < P; j0 += BJ) {
+        double acc[2][4] = {};
+        for (int i0 = 0; i0 < P; i0 += BI) {
+            __syncthreads();
+            for (int e = tid; e < BI * BR; e += 256) {
+                const int r = e / BI, i = e % BI;
+                As[i][r] = (k0 + r < P && i0 + i < P) ? X[(size_t)(k0 + r) * P + i0 + i] : 0.0;
+            }
+            for (int e = tid; e < BI * BJ; e += 256) {
+                // (along the stored row on either side of the diagonal)
+                const bool below = i0 >= j0 + BJ;
+                const int i = below ? e % BI : e / BJ, j = below ? e / BI : e % BJ;
+                const int a = min(i0 + i, j0 + j), b = max(i0 + i, j0 + j);
+                Bs[i][j] = b < P ? M[(size_t)a * P + b] : 0.0;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < BI; ++i)
+#pragma unroll
+                for (int a = 0; a < 2; ++a)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) acc[a][b] = fma(As[i][2 * ty + a], Bs[i][tx + 16 * b], acc[a][b]);
+        }
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const int k = k0 + 2 * ty + a, j = j0 + tx + 16 * b;
+                if (k < P && j < P) q2[a] = fma(acc[a][b], X[(size_t)k * P + j], q2[a]);
+            }
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+#pragma unroll
+        for (int off = 8; off > 0; off >>= 1) q2[a] += __shfl_xor_sync(0xffffffffu, q2[a], off);
+        const int k = k0 + 2 * ty + a;
+        if (tx == 0 && k < P) SnrScratch{M, P}.e(k) = q2[a];
+    }
+}
+
+// ------------------------------------------------------------------------------ the solution
+__global__ void __launch_bounds__(256) snr_final_kernel(int P, int ns, const double2* __restrict__ D, double thr,
+                                                        double eps_svd, double* Aws, const double* __restrict__ Xws,
+                                                        double2* __restrict__ delta, double* __restrict__ lam_out) {
+    const int t = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    extern __shared__ __align__(16) double sm[];
+    double2* cf = reinterpret_cast<double2*>(sm);  // [P] filtered coefficients
+    __shared__ double red[8];
+    const double* X = Xws + (size_t)t * P * P;
+    const SnrScratch sc{Aws + (size_t)t * P * P, P};  // eigenvalue and v^T M v
+    double2* xt = delta + (size_t)t * P;
+    const double2* Dt = D + (size_t)t * P;
+    double lm = -INFINITY;
+    int bad = 0;
+    for (int k = tid; k < P; k += 256) {
+        lm = fmax(lm, sc.d(k));
+        bad |= isnan(sc.d(k));
+    }
+    bad = __syncthreads_or(bad);
+    if (bad) {
+        for (int k = tid; k < P; k += 256) xt[k] = make_double2(0.0, 0.0);
         return;
     }
-
-    // ---- (4) rho = V^T D (row k of X is eigenvector k), mean of v
-    double2* rho = reinterpret_cast<double2*>(tau);  // tau and vb: P double2
-    double2* qs = reinterpret_cast<double2*>(pb);    // pb and cs: sum of Q_k
-    double* q2 = ss;                                 // sum of |Q_k|^2
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) lm = fmax(lm, __shfl_xor_sync(0xffffffffu, lm, off));
+    if (lane == 0) red[warp] = lm;
     __syncthreads();
-    const double2* Dt = D + (size_t)t * P;
-    for (int k = warp; k < P; k += SNRB_WARPS) {
+    lm = red[0];
+    for (int i = 1; i < 8; ++i) lm = fmax(lm, red[i]);
+    for (int k = warp; k < P; k += 8) {
         const double* Xk = X + (size_t)k * P;
         double ax = 0.0, ay = 0.0;
+#pragma unroll 4
         for (int i = lane; i < P; i += 32) {
             ax += Xk[i] * Dt[i].x;
             ay += Xk[i] * Dt[i].y;
         }
-        ax = warp_sum(ax);
+        ax = warp_sum(ax);  // rho_k
         ay = warp_sum(ay);
         if (lane == 0) {
-            rho[k] = make_double2(ax, ay);
-            qs[k] = make_double2(0.0, 0.0);
-            q2[k] = 0.0;
+            const double lam = sc.d(k), r2 = ax * ax + ay * ay;
+            const double var = fmax(sc.e(k) / ns - r2, 0.0);
+            const double snr = sqrt(r2) / sqrt(var / ns + 1e-300);
+            const double f_snr = 1.0 / (1.0 + pow(thr / snr, 6.0));
+            const double f_svd = 1.0 / (1.0 + pow(eps_svd * lm / fmax(lam, 1e-300), 6.0));
+            const double inv = lam > 0.0 ? f_snr * f_svd / fmax(lam, 1e-300) : 0.0;
+            cf[k] = make_double2(inv * ax, inv * ay);
+            if (lam_out) lam_out[(size_t)t * P + k] = lam;
         }
     }
-    const double2* vt = v + (size_t)t * ns;
-    double sx = 0.0, sy = 0.0;
-    for (int x = tid; x < ns; x += blockDim.x) {
-        sx += vt[x].x;
-        sy += vt[x].y;
-    }
-    const double vbx = block_sum(sx, red) / ns;
-    const double vby = block_sum(sy, red) / ns;
     __syncthreads();
-
-    // one pass over the samples in chunks: y_k(x) = sum_i V_ik O_c,i(x), Q = y v_c
-    const int CH = snrb_chunk(P);
-    const uint64_t* sp = spins + (size_t)t * ns * W;
-    const double* ob = obar + (size_t)t * P;
-    const int16_t* Ot = Oint != nullptr ? Oint + (size_t)t * P * ns : nullptr;
-    if (fp32_pass) {
-        // y in FP32 from an FP32 copy of the eigenvectors (in A's place, no longer needed):
-        // the variances only set the filter, to a relative accuracy of about 1e-6
-        float* Xf = reinterpret_cast<float*>(A);
-        for (size_t i = tid; i < PP; i += blockDim.x) Xf[i] = (float)X[i];
-        __syncthreads();
-        snrb_sample_pass<float>(n, W, P, ns, sp, pairs, grp_off, grp_pair, Ot, ob, Xf, reinterpret_cast<float*>(och),
-                                sgn, CH, vt, vbx, vby, qs, q2);
-    } else {
-        snrb_sample_pass<double>(n, W, P, ns, sp, pairs, grp_off, grp_pair, Ot, ob, X, och, sgn, CH, vt, vbx, vby, qs,
-                                 q2);
-    }
-
-    // ---- (5) filter and back-projection: delta_i = sum_k V_ik c_k, c_k = f_k rho_k / lambda_k
-    double lm = -INFINITY;
-    for (int k = tid; k < P; k += blockDim.x) lm = fmax(lm, d[k]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) lm = fmax(lm, __shfl_xor_sync(0xffffffffu, lm, off));
-    __syncthreads();
-    if (lane == 0) red[warp] = lm;
-    __syncthreads();
-    lm = red[0];
-    for (int i = 1; i < SNRB_WARPS; ++i) lm = fmax(lm, red[i]);
-    // the filtered coefficients go to the chunk buffer (2 P doubles at least), clear of rho/qs/q2
-    double2* cf = reinterpret_cast<double2*>(och);
-    for (int k = tid; k < P; k += blockDim.x) {
-        const double lam = d[k];
-        const double mqx = qs[k].x / ns, mqy = qs[k].y / ns;
-        const double var = fmax(q2[k] / ns - (mqx * mqx + mqy * mqy), 0.0);
-        const double snr = sqrt(rho[k].x * rho[k].x + rho[k].y * rho[k].y) / sqrt(var / ns + 1e-300);
-        const double f_snr = 1.0 / (1.0 + pow(thr / snr, 6.0));
-        const double f_svd = 1.0 / (1.0 + pow(eps_svd * lm / fmax(lam, 1e-300), 6.0));
-        const double inv = lam > 0.0 ? f_snr * f_svd / fmax(lam, 1e-300) : 0.0;
-        cf[k] = make_double2(inv * rho[k].x, inv * rho[k].y);
-        if (lam_out) lam_out[(size_t)t * P + k] = lam;
-    }
-    __syncthreads();
-    for (int i = tid; i < P; i += blockDim.x) {
+    for (int i = tid; i < P; i += 256) {
         double ax = 0.0, ay = 0.0;
+#pragma unroll 4
         for (int k = 0; k < P; ++k) {
             const double xki = X[(size_t)k * P + i];
             ax += xki * cf[k].x;
             ay += xki * cf[k].y;
         }
-        delta[(size_t)t * P + i] = make_double2(ax, ay);
+        xt[i] = make_double2(ax, ay);
     }
 }
 
-size_t snr_big_smem_bytes(int P) {
-    return (size_t)(7 * P + 32 + (P & 1) + snrb_chunk(P) * P) * sizeof(double) + SNRB_SGN_BYTES;
+size_t snr_big_ws_bytes(int ntraj, int P) {
+    return (size_t)ntraj * 2 * (size_t)P * P * sizeof(double) + 256;
 }
 
-size_t snr_big_ws_bytes(int ntraj, int P) { return (size_t)ntraj * 2 * (size_t)P * P * sizeof(double) + 256; }
-
-bool snr_big_fits(int P) { return snrb_chunk(P) >= 2; }
+// (the bound of the one-kernel form, kept: about P = 3000)
+bool snr_big_fits(int P) { return (SNRB_SMEM_BUDGET / 8 - 7 * P - 33) / P >= 2; }
 
 cudaError_t launch_snr_big(const otvmc_ansatz* a, int ntraj, int ns, const uint64_t* spins, const double* S,
                            const double* obar, const double2* v, const double2* D, double thr, double eps_svd,
-                           double2* delta, double* lam, void* ws, int* status, cudaStream_t s, bool fp32_pass,
-                           const int16_t* Oint) {
+                           double2* delta, double* lam, void* ws, int* status, cudaStream_t s) {
     ProfScope prof_(OTVMC_K_SOLVE, s);
-    const int P = (int)a->P, n = a->n, W = (n + 63) / 64;
-    const size_t smem = snr_big_smem_bytes(P);
-    cudaError_t e = cudaFuncSetAttribute(snr_big_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    const int P = (int)a->P, n = a->n;
     double* Aws = (double*)ws;
     double* Xws = Aws + (size_t)ntraj * P * P;
     const bool tied = a->kind == OTVMC_LJ;
-    snr_big_kernel<<<ntraj, SNRB_THREADS, smem, s>>>(n, W, P, ns, spins, tied ? a->full->pairs_d : a->pairs_d,
-                                                     tied ? a->grp_off_d : nullptr, tied ? a->grp_pair_d : nullptr,
-                                                     S, obar, v, D, thr, eps_svd, Aws, Xws, delta, lam, status,
-                                                     fp32_pass ? 1 : 0, Oint);
-    count_launch();
+    const OShape o{n, (n + 63) / 64, P, tied ? n + a->nfree : P, tied ? a->lj_d : 0, tied ? a->lj_pbc : 0,
+                   tied ? a->full->pairs_d : a->pairs_d, tied ? a->grp_pair_d : nullptr};
+    const int smem_tri = (5 * P + SNRB_WARPS) * (int)sizeof(double), smem_ql = 6 * P * (int)sizeof(double);
+    cudaError_t e = cudaFuncSetAttribute(snr_tri_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_tri);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(snr_ql_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_ql);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(snr_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * P * (int)sizeof(double));
+    if (e != cudaSuccess) return e;
+    const int nt = (P + WG - 1) / WG;
+    snr_tri_kernel<<<ntraj, SNRB_THREADS, smem_tri, s>>>(P, S, Aws, Xws);
+    snr_wgram_kernel<<<dim3(nt * (nt + 1) / 2, ntraj), 256, 0, s>>>(o, ns, spins, v, obar, Aws);
+    snr_ql_kernel<<<ntraj, 32 + QL_APPLY, smem_ql, s>>>(P, Aws, Xws, status);
+    snr_var_kernel<<<dim3((P + 31) / 32, ntraj), 256, 0, s>>>(P, Xws, Aws);
+    snr_final_kernel<<<ntraj, 256, 2 * P * (int)sizeof(double), s>>>(P, ns, D, thr, eps_svd, Aws, Xws, delta, lam);
+    count_launch(5);
     return cudaGetLastError();
 }
 
