@@ -24,7 +24,8 @@
 // Bound: FP64 at 2 multiply-adds per cycle and SM (tri: about 5/3 P^3 of them, ql: 2 per rotation and
 // column, about 3 P^3, var: P^3), and in ql the chain of the recurrence (about 0.85 P^2 rotations).
 // 100 trajectories of P = 249, 4096 samples, in one kernel with FP64 projections of every sample
-// and the recurrence between the rotations: 321 ms; now 85 ms (tri 18, wgram 10, ql 53, var 3).
+// and the recurrence between the rotations: 321 ms; now 70 ms (tri
+// 12, wgram 8, ql 47, var 3; ql at 1,700 cycles a rotation of its recurrence, 730 of its columns).
 // A and X live in the caller's workspace (2 P^2 doubles per trajectory).  Only the upper triangle of M
 // is stored; d, e and v^T M v pass from launch to launch in the lower one (SnrScratch).
 #include "common.cuh"
@@ -40,6 +41,36 @@ __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     return v;
+}
+
+// Sums over the 32 lanes of eight values per lane in 9 additions (each step halves the values a lane
+// keeps; additions are what an FP64 reduction costs); every lane gets all eight totals.
+__device__ __forceinline__ void warp_sum8(double (&v)[8]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int h = 4, off = 16; h >= 1; h >>= 1, off >>= 1) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (u < h) {
+                const double send = up ? v[u] : v[u + h], keep = up ? v[u + h] : v[u];
+                v[u] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+            }
+    }
+    double s = v[0];
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    // lane bits 4, 3, 2 hold the index of its total
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+        v[u] = __shfl_sync(0xffffffffu, s, ((u >> 2) & 1) * 16 + ((u >> 1) & 1) * 8 + (u & 1) * 4);
+}
+
+__device__ __forceinline__ double pick8(const double (&v)[8], int i) {
+    double r = v[0];
+#pragma unroll
+    for (int u = 1; u < 8; ++u) r = i == u ? v[u] : r;
+    return r;
 }
 
 // Sum over a CTA of NW warps (every thread calls it; red holds NW doubles).
@@ -107,14 +138,19 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_tri_kernel(int P, const d
         }
         __syncthreads();
         if (tk != 0.0) {
-            // p = tau B v (B the trailing block), one warp per row
-            for (int i = warp; i < m; i += SNRB_WARPS) {
-                const double* Bi = A + (size_t)(k + 1 + i) * P + k + 1;
-                double s = 0.0;
-#pragma unroll 8
-                for (int j = lane; j < m; j += 32) s += Bi[j] * vb[j];
-                s = warp_sum(s);
-                if (lane == 0) pb[i] = tk * s;
+            // p = tau B v (B the trailing block), eight rows per warp
+            for (int i0 = 8 * warp; i0 < m; i0 += 8 * SNRB_WARPS) {
+                const double* Bi = A + (size_t)(k + 1 + i0) * P + k + 1;
+                const int nr = min(8, m - i0);
+                double s[8] = {};
+                for (int j = lane; j < m; j += 32) {
+                    const double vj = vb[j];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (u < nr) s[u] = fma(Bi[(size_t)u * P + j], vj, s[u]);
+                }
+                warp_sum8(s);
+                if (lane < nr) pb[i0 + lane] = tk * pick8(s, lane);
             }
             __syncthreads();
             double pv = 0.0;
@@ -123,11 +159,24 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_tri_kernel(int P, const d
             for (int i = tid; i < m; i += blockDim.x) pb[i] -= K * vb[i];  // w = p - K v
             __syncthreads();
             // B -= v w^T + w v^T
-            for (int i = warp; i < m; i += SNRB_WARPS) {
-                double* Bi = A + (size_t)(k + 1 + i) * P + k + 1;
-                const double vi = vb[i], wi = pb[i];
-#pragma unroll 8
-                for (int j = lane; j < m; j += 32) Bi[j] -= vi * pb[j] + wi * vb[j];
+            for (int i0 = 8 * warp; i0 < m; i0 += 8 * SNRB_WARPS) {
+                double* Bi = A + (size_t)(k + 1 + i0) * P + k + 1;
+                const int nr = min(8, m - i0);
+                double vi[8], wi[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    vi[u] = u < nr ? -vb[i0 + u] : 0.0;
+                    wi[u] = u < nr ? -pb[i0 + u] : 0.0;
+                }
+                for (int j = lane; j < m; j += 32) {
+                    const double pj = pb[j], vj = vb[j];
+                    double x[8];
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) x[u] = u < nr ? Bi[(size_t)u * P + j] : 0.0;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u)
+                        if (u < nr) Bi[(size_t)u * P + j] = fma(vi[u], pj, fma(wi[u], vj, x[u]));
+                }
             }
         }
         __syncthreads();
@@ -154,15 +203,29 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_tri_kernel(int P, const d
         for (int i = tid; i < m; i += blockDim.x) vb[i] = A[(size_t)(k + 1 + i) * P + k];
         __syncthreads();
         // rows r >= k + 1 of X are the only ones with entries in columns k + 1 .. (X is the
-        // identity elsewhere): u_r = (X v)_r, then X[r][k+1+b] -= tau u_r v_b, a warp per row
-        for (int r = warp; r < m; r += SNRB_WARPS) {
-            double* Xr = X + (size_t)(k + 1 + r) * P + k + 1;
-            double s = 0.0;
-#pragma unroll 8
-            for (int b = lane; b < m; b += 32) s += Xr[b] * vb[b];
-            const double u = tk * warp_sum(s);
-#pragma unroll 8
-            for (int b = lane; b < m; b += 32) Xr[b] -= u * vb[b];
+        // identity elsewhere): u_r = (X v)_r, then X[r][k+1+b] -= tau u_r v_b, eight rows per warp
+        for (int r0 = 8 * warp; r0 < m; r0 += 8 * SNRB_WARPS) {
+            double* Xr = X + (size_t)(k + 1 + r0) * P + k + 1;
+            const int nr = min(8, m - r0);
+            double s[8] = {};
+            for (int b = lane; b < m; b += 32) {
+                const double v = vb[b];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (u < nr) s[u] = fma(Xr[(size_t)u * P + b], v, s[u]);
+            }
+            warp_sum8(s);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s[u] *= -tk;
+            for (int b = lane; b < m; b += 32) {
+                const double v = vb[b];
+                double x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) x[u] = u < nr ? Xr[(size_t)u * P + b] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (u < nr) Xr[(size_t)u * P + b] = fma(s[u], v, x[u]);
+            }
         }
         __syncthreads();
     }
@@ -223,7 +286,7 @@ __device__ __forceinline__ double to_double(__int128 v) {
 }
 
 // The upper triangle of M, a 64 x 64 tile per CTA.
-__global__ void __launch_bounds__(256) snr_wgram_kernel(OShape o, int ns, const uint64_t* __restrict__ spins,
+__global__ void __launch_bounds__(256, 2) snr_wgram_kernel(OShape o, int ns, const uint64_t* __restrict__ spins,
                                                         const double2* __restrict__ v,
                                                         const double* __restrict__ obar, double* __restrict__ M) {
     const int t = blockIdx.y, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
@@ -370,9 +433,32 @@ __global__ void __launch_bounds__(256) snr_wgram_kernel(OShape o, int ns, const 
 }
 
 // --------------------------------------------------------------------------- QL iteration
-constexpr int QL_APPLY = 256;  // threads that apply rotations, a column of X each
+// Twelve warps, of which warp 0 runs the recurrence and the nine that do not share its scheduler apply
+// rotations, a column of X per thread: an FP64 instruction holds a scheduler's FP64 unit for 64
+// cycles whatever the number of its lanes, so the recurrence costs what it counts in FP64
+// instructions (19 a rotation, with comparisons, doublings and the first approximation of the
+// reciprocal root in integers and FP32).
+constexpr int QL_THREADS = 384;
+constexpr int QL_APPLY = 288;
 
-__global__ void __launch_bounds__(32 + QL_APPLY, 1) snr_ql_kernel(int P, double* __restrict__ Aws,
+// 1 / sqrt(h) for a normal positive h: FP32 approximation y (2^-22) of the root of h's mantissa, then
+// one step of third order, y + y e (1/2 + 3/8 e) with e = 1 - h y^2.
+__device__ __forceinline__ double rsqrt_pos(double h) {
+    const int hw = __double2hiint(h), lw = __double2loint(h);
+    const int E = (hw >> 20) - 1023, k = E >> 1;  // h = mantissa 2^(E & 1) 2^(2 k)
+    const float m = __int_as_float(((127 + (E & 1)) << 23) | ((hw & 0xFFFFF) << 3) | (int)((unsigned)lw >> 29));
+    const int yb = __float_as_int(rsqrtf(m));
+    const double y = __hiloint2double((((yb >> 23) + 896 - k) << 20) | ((yb & 0x7FFFFF) >> 3), yb << 29);
+    const double e = fma(-(h * y), y, 1.0);
+    return fma(y * e, fma(0.375, e, 0.5), y);
+}
+// 2 x for a normal x, and 0 for 0
+__device__ __forceinline__ double twice(double x) {
+    const int hw = __double2hiint(x);
+    return (hw & 0x7FF00000) ? __hiloint2double(hw + 0x100000, __double2loint(x)) : x;
+}
+
+__global__ void __launch_bounds__(QL_THREADS, 1) snr_ql_kernel(int P, double* __restrict__ Aws,
                                                                   double* __restrict__ Xws, int* status) {
     const int t = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     extern __shared__ __align__(16) double sm[];
@@ -443,24 +529,26 @@ __global__ void __launch_bounds__(32 + QL_APPLY, 1) snr_ql_kernel(int P, double*
                     const double f = s * ei, b = c * ei;
                     const double h2 = fma(f, f, g * g);
                     double ir;
-                    if (h2 > 1e-290) {
-                        ir = rsqrt(h2);
+                    const int ex = __double2hiint(h2) >> 20;
+                    if (ex > 64 && ex < 2000) {
+                        ir = rsqrt_pos(h2);
                         r = h2 * ir;
-                    } else {  // squares below the normal range
+                    } else {  // squares near or below the normal range (or not finite)
                         r = hypot(f, g);
                         ir = r > 0.0 ? 1.0 / r : 0.0;
+                        if (r == 0.0) {  // deflation inside the sweep
+                            e[i + 1] = 0.0;
+                            d[i + 1] = dn - p;
+                            e[m] = 0.0;
+                            underflow = true;
+                            break;
+                        }
                     }
                     e[i + 1] = r;
-                    if (r == 0.0) {  // deflation inside the sweep
-                        d[i + 1] = dn - p;
-                        e[m] = 0.0;
-                        underflow = true;
-                        break;
-                    }
                     s = f * ir;
                     c = g * ir;
                     g = dn - p;
-                    r = fma(di - g, s, 2.0 * c * b);
+                    r = fma(twice(c), b, (di - g) * s);
                     p = s * r;
                     d[i + 1] = g + p;
                     g = fma(c, r, -b);
@@ -484,12 +572,12 @@ __global__ void __launch_bounds__(32 + QL_APPLY, 1) snr_ql_kernel(int P, double*
                 if (fail) sm_fail = 1;
             }
             __syncwarp();
-        } else if (step > 0) {
+        } else if (step > 0 && (warp & 3) != 0) {
             // rotations i = m - 1 down to lo of the sweep before, on rows i and i + 1 of every column
             const int buf = (step - 1) & 1, m = sm_m[buf], lo = sm_lo[buf];
             const double *cs = cs2 + buf * P, *ss = ss2 + buf * P;
             if (m - 1 >= lo)
-                for (int col = tid - 32; col < P; col += QL_APPLY) {
+                for (int col = 32 * (3 * (warp >> 2) + (warp & 3) - 1) + lane; col < P; col += QL_APPLY) {
                     double zi1 = X[(size_t)m * P + col];  // row i + 1 for i = m - 1
                     // rows are loaded ahead of the rotations that use them (each row is stored only
                     // after it has been loaded)
@@ -660,7 +748,7 @@ cudaError_t launch_snr_big(const otvmc_ansatz* a, int ntraj, int ns, const uint6
     const int nt = (P + WG - 1) / WG;
     snr_tri_kernel<<<ntraj, SNRB_THREADS, smem_tri, s>>>(P, S, Aws, Xws);
     snr_wgram_kernel<<<dim3(nt * (nt + 1) / 2, ntraj), 256, 0, s>>>(o, ns, spins, v, obar, Aws);
-    snr_ql_kernel<<<ntraj, 32 + QL_APPLY, smem_ql, s>>>(P, Aws, Xws, status);
+    snr_ql_kernel<<<ntraj, QL_THREADS, smem_ql, s>>>(P, Aws, Xws, status);
     snr_var_kernel<<<dim3((P + 31) / 32, ntraj), 256, 0, s>>>(P, Xws, Aws);
     snr_final_kernel<<<ntraj, 256, 2 * P * (int)sizeof(double), s>>>(P, ns, D, thr, eps_svd, Aws, Xws, delta, lam);
     count_launch(5);
