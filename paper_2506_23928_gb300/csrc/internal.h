@@ -299,6 +299,19 @@ size_t obs_tc_bytes(int ntraj, int n);
 cudaError_t obs_tc_set_wait_limit(unsigned long long ns);
 cudaError_t launch_obs_tc(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,
                           double* moments, int* status, cudaStream_t s);
+// Wide chains on the mixed path (k_wide.cu): estimators beyond the tensor-core kernel's sites and
+// observables beyond theirs.  From about two samples per site the records of the estimators fit
+// the half of b.r that FP32 ratios leave free; below that the general kernel stays.
+bool est_wide_ok(const otvmc_ansatz* a, bool fp32, int ntraj, int ns);
+cudaError_t launch_est1_wide(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,
+                             cudaStream_t s);
+cudaError_t launch_obs_prep_wide(const otvmc_ansatz* a, const double2* theta, int ntraj, const EvalBufs& b,
+                                 cudaStream_t s);
+cudaError_t launch_obs_wide(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,
+                            double* moments, cudaStream_t s);
+inline bool obs_wide_ok(const otvmc_ansatz* a, bool fp32) {
+    return fp32 && a->kind == OTVMC_JASTROW && a->n > OTC_MAX_N;
+}
 inline bool obs_tc_ok(const otvmc_ansatz* a, bool fp32) {
     return fp32 && a->kind == OTVMC_JASTROW && a->n >= OTC_MIN_N && a->n <= OTC_MAX_N;
 }

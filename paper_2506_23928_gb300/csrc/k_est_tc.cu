@@ -21,7 +21,9 @@
 // SIMT path.  The real fields carry FP32-level rounding.
 //
 // One CTA = 16 sites x 4 tiles of 128 samples of one trajectory, 128 threads (one per sample
-// of a tile), 128 TMEM columns, so that four CTAs share an SM:
+// of a tile), 128 TMEM columns, so that four CTAs share an SM at N <= 64 and three
+// beyond (32 KB of operands per 64 sites; beyond 64 sites the tile's ratios take the place of
+// the sigma tile, whose products are done; with 16 KB of their own two CTAs fit):
 //   - the B image of the site block (8 x 16 rows of 64 k per 64-site block kb, pre-swizzled
 //     by est_tc_prep_kernel) arrives by one bulk copy;
 //   - per tile every thread writes its sample's row of the sigma tile into shared memory
@@ -163,19 +165,22 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+template <int KB>
 struct Smem {
     uint64_t bfull, mma;
     uint32_t tmem_slot;
     int abort_flag;
-    float2 rs[SB][128];       // the tile's ratios, site-major
-    uint64_t sw[2][128];      // the tile's spin words (64-site blocks 0 and 1)
+    uint64_t sw[KB][128];     // the tile's spin words, by 64-site block
     float tab[4][SB];         // aRe, sRe, aJ, sJ of the block's sites
     long long aim[SB];
     double acc[SB][5];        // per site: sums of Re r, Im r, sigma Re r, sigma Im r, sigma
 };
 
+// CTAs per SM: by TMEM for KB = 1, by shared memory beyond
+constexpr int ctas_per_sm(int KB) { return KB == 1 ? 4 : 3; }
+
 template <int KB>
-__global__ void __launch_bounds__(128, 4) est_tc_kernel(int n, int ns, double h, const uint64_t* __restrict__ spins,
+__global__ void __launch_bounds__(128, ctas_per_sm(KB)) est_tc_kernel(int n, int ns, double h, const uint64_t* __restrict__ spins,
                                                         const uint8_t* __restrict__ img, SiteTabs tabs,
                                                         float2* __restrict__ r_out, double2* __restrict__ EHq,
                                                         double2* __restrict__ part_r, double2* __restrict__ part_sr,
@@ -184,7 +189,10 @@ __global__ void __launch_bounds__(128, 4) est_tc_kernel(int n, int ns, double h,
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sA = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint8_t* sB = sA + KB * A_BYTES;
-    Smem& S = *reinterpret_cast<Smem*>(sB + KB * B_BYTES);
+    Smem<KB>& S = *reinterpret_cast<Smem<KB>*>(sB + KB * B_BYTES);
+    // the tile's ratios, site-major: behind the rest for KB = 1, else over the sigma tile (written
+    // once the tile's products are complete, read before the next tile's rows are written)
+    float2(*rs)[128] = reinterpret_cast<float2(*)[128]>(KB == 1 ? (uint8_t*)(&S + 1) : sA);
     const int chunk = blockIdx.x, sb = blockIdx.y, t = blockIdx.z, nsb = gridDim.y;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int W = (n + 63) / 64;
@@ -233,21 +241,14 @@ __global__ void __launch_bounds__(128, 4) est_tc_kernel(int n, int ns, double h,
         for (int kb = 0; kb < KB; ++kb) {
             const uint64_t word = sv ? spins[((size_t)t * ns + s) * W + kb] : 0ull;
             S.sw[kb][tid] = word;
+            // (bits beyond the last site meet zero rows of B, and rows beyond the last sample are not read)
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
+                const uint32_t x = (uint32_t)(word >> (8 * c));
                 uint32_t w4[4];
 #pragma unroll
-                for (int e2 = 0; e2 < 4; ++e2) {
-                    uint32_t v2 = 0;
-#pragma unroll
-                    for (int e1 = 0; e1 < 2; ++e1) {
-                        const int e = 2 * e2 + e1, k = 64 * kb + 8 * c + e;
-                        const uint32_t bit = (uint32_t)(word >> (8 * c + e)) & 1u;
-                        const uint32_t code = (sv && k < n) ? (0xBC00u ^ (bit << 15)) : 0u;
-                        v2 |= code << (16 * e1);
-                    }
-                    w4[e2] = v2;
-                }
+                for (int i = 0; i < 4; ++i)  // 0xBC00 = -1, the sign cleared where the bit is set
+                    w4[i] = 0xBC00BC00u ^ ((x << (15 - 2 * i)) & 0x8000u) ^ ((x << (30 - 2 * i)) & 0x80000000u);
                 *reinterpret_cast<uint4*>(sA + kb * A_BYTES + sw128(tid, c)) = make_uint4(w4[0], w4[1], w4[2], w4[3]);
             }
         }
@@ -259,12 +260,12 @@ __global__ void __launch_bounds__(128, 4) est_tc_kernel(int n, int ns, double h,
             if (ok) {
                 fence_after();
                 constexpr uint32_t ID = idesc_f16(128, NCOL);
-#pragma unroll
-                for (int kb = 0; kb < KB; ++kb)
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        umma(tmem, smem_desc(su32(sA + kb * A_BYTES) + k * 32), smem_desc(su32(sB + kb * B_BYTES) + k * 32),
-                             ID, (kb > 0 || k > 0) ? 1u : 0u);
+                const int ksteps = (n + 15) / 16;
+                for (int k = 0; k < ksteps; ++k) {
+                    const int kb = k >> 2, off = (k & 3) * 32;
+                    umma(tmem, smem_desc(su32(sA + kb * A_BYTES) + off), smem_desc(su32(sB + kb * B_BYTES) + off), ID,
+                         k > 0 ? 1u : 0u);
+                }
                 umma_commit(&S.mma);
                 ++issued;
             } else {
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(128, 4) est_tc_kernel(int n, int ns, double h,
                         hrx += rr[u].x;
                         hry += rr[u].y;
                     }
-                    S.rs[8 * g + u][tid] = rr[u];
+                    rs[8 * g + u][tid] = rr[u];
                 }
                 if (sv) {
                     const int j0 = jb0 + 8 * g;
@@ -359,7 +360,7 @@ __global__ void __launch_bounds__(128, 4) est_tc_kernel(int n, int ns, double h,
             float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, a4 = 0.f;
 #pragma unroll 4
             for (int i = p; i < 128; i += 8) {
-                const float2 r = S.rs[u][i];
+                const float2 r = rs[u][i];
                 const bool in = s0 + i < ns && jb0 + u < n;
                 const float sg = in ? (((S.sw[kw][i] >> sh) & 1ull) ? 1.f : -1.f) : 0.f;
                 a0 += r.x;
@@ -411,7 +412,7 @@ __global__ void __launch_bounds__(128, 4) est_tc_kernel(int n, int ns, double h,
 
 template <int KB>
 constexpr int smem_bytes() {
-    return KB * (A_BYTES + B_BYTES) + (int)sizeof(Smem) + 1024;
+    return KB * (A_BYTES + B_BYTES) + (int)sizeof(Smem<KB>) + (KB == 1 ? SB * 128 * 8 : 0) + 1024;
 }
 
 }  // namespace etc
@@ -446,21 +447,17 @@ cudaError_t launch_est_tc(const otvmc_ansatz* a, const uint64_t* spins, int ntra
     if (e != cudaSuccess) return e;
     const int nblk = est_tc_chunks(ns);
     dim3 grid(nblk, nsb, ntraj);
-    if (KB == 1) {
-        constexpr int SM = etc::smem_bytes<1>();
-        e = cudaFuncSetAttribute(etc::est_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
-        if (e != cudaSuccess) return e;
-        etc::est_tc_kernel<1><<<grid, 128, SM, s>>>(n, ns, m->h, spins, img, tabs,
-                                                    reinterpret_cast<float2*>(b.r), b.EH, b.part_r, b.part_sr,
-                                                    b.part_s, nblk, status);
-    } else {
-        constexpr int SM = etc::smem_bytes<2>();
-        e = cudaFuncSetAttribute(etc::est_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);
-        if (e != cudaSuccess) return e;
-        etc::est_tc_kernel<2><<<grid, 128, SM, s>>>(n, ns, m->h, spins, img, tabs,
-                                                    reinterpret_cast<float2*>(b.r), b.EH, b.part_r, b.part_sr,
-                                                    b.part_s, nblk, status);
-    }
+#define OTVMC_EST_TC_LAUNCH(K)                                                                                    \
+    do {                                                                                                          \
+        constexpr int SM = etc::smem_bytes<K>();                                                                  \
+        e = cudaFuncSetAttribute(etc::est_tc_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);         \
+        if (e != cudaSuccess) return e;                                                                           \
+        etc::est_tc_kernel<K><<<grid, 128, SM, s>>>(n, ns, m->h, spins, img, tabs, reinterpret_cast<float2*>(b.r), \
+                                                    b.EH, b.part_r, b.part_sr, b.part_s, nblk, status);           \
+    } while (0)
+    if (KB == 1) OTVMC_EST_TC_LAUNCH(1);
+    else OTVMC_EST_TC_LAUNCH(2);
+#undef OTVMC_EST_TC_LAUNCH
     count_launch();
     return cudaGetLastError();
 }

@@ -282,6 +282,7 @@ static size_t est1_smem(int n, int W) {
 cudaError_t launch_est1_jastrow(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, bool fp32,
                                 const EvalBufs& b, int* status, cudaStream_t s) {
     if (est_tc_ok(a, fp32)) return launch_est_tc(a, spins, ntraj, ns, b, status, s);
+    if (est_wide_ok(a, fp32, ntraj, ns)) return launch_est1_wide(a, spins, ntraj, ns, b, s);
     ProfScope prof_(OTVMC_K_EST1, s);
     (void)status;
     const int n = a->n, W = (n + 63) / 64;
@@ -675,7 +676,7 @@ __global__ void obs_prep_kernel(const double2* __restrict__ theta, int P, int n,
 cudaError_t launch_obs_prep(const otvmc_ansatz* a, const double2* theta, int ntraj, bool fp32, const EvalBufs& b,
                             cudaStream_t s) {
     ProfScope prof_(OTVMC_K_OBS, s);
-    (void)fp32;
+    if (obs_wide_ok(a, fp32)) return launch_obs_prep_wide(a, theta, ntraj, b, s);
     obs_prep_kernel<<<ntraj, 256, 0, s>>>(theta, (int)a->P, a->n, b.Epm);
     count_launch();
     return cudaGetLastError();
@@ -814,6 +815,7 @@ cudaError_t launch_obs_final(int n, int ns, int ntraj, const EvalBufs& b, double
 cudaError_t launch_observables(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, bool fp32,
                                const EvalBufs& b, double* moments, int* status, cudaStream_t s) {
     if (obs_tc_ok(a, fp32) && b.otc != nullptr) return launch_obs_tc(a, spins, ntraj, ns, b, moments, status, s);
+    if (obs_wide_ok(a, fp32)) return launch_obs_wide(a, spins, ntraj, ns, b, moments, s);
     ProfScope prof_(OTVMC_K_OBS, s);
     const int n = a->n, W = (n + 63) / 64;
     const int NT = ((n + 31) / 32) * 32, SPP = 256 / NT;
@@ -835,8 +837,7 @@ cudaError_t launch_observables(const otvmc_ansatz* a, const uint64_t* spins, int
                                                              reinterpret_cast<const R2*>(b.r), b.Epm, b.part_obs);  \
     } while (0)
     if (fp32) {
-        if (sm) OTVMC_OBS_LAUNCH(float2, float, true);
-        else OTVMC_OBS_LAUNCH(float2, float, false);
+        OTVMC_OBS_LAUNCH(float2, float, true);  // below OTC_MIN_N sites: the tables fit
     } else {
         if (sm) OTVMC_OBS_LAUNCH(double2, double, true);
         else OTVMC_OBS_LAUNCH(double2, double, false);
