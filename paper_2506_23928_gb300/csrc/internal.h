@@ -300,7 +300,7 @@ cudaError_t obs_tc_set_wait_limit(unsigned long long ns);
 cudaError_t launch_obs_tc(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,
                           double* moments, int* status, cudaStream_t s);
 // Wide chains on the mixed path (k_wide.cu): estimators beyond the tensor-core kernel's sites and
-// observables beyond theirs.  From about two samples per site the records of the estimators fit
+// observables beyond theirs.  From about a sample per site the records of the estimators fit
 // the half of b.r that FP32 ratios leave free; below that the general kernel stays.
 bool est_wide_ok(const otvmc_ansatz* a, bool fp32, int ntraj, int ns);
 cudaError_t launch_est1_wide(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,

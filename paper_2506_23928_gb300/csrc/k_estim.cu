@@ -305,35 +305,39 @@ cudaError_t launch_est1_jastrow(const otvmc_ansatz* a, const uint64_t* spins, in
 }
 
 // -------------------------------------------------------------------- site means, <L+L^+>
-// mean_r_j = <r_j> (local sx_j), mean_sr_j = <sigma_j r_j>, mean_s_j = <sigma_j>; then
-// <L + L^+> = sqrt(kappa_j) Re mean_r_j (decay), 2 sqrt(gamma_j) mean_s_j (dephasing).
-__global__ void site_means_kernel(int n, int nblk, int ns, int nops, const double2* __restrict__ part_r,
-                                  const double2* __restrict__ part_sr, const double* __restrict__ part_s,
-                                  const double* __restrict__ site, const int* __restrict__ opidx,
-                                  double2* __restrict__ mean_r, double2* __restrict__ mean_sr,
-                                  double* __restrict__ mean_s, double* __restrict__ lpl) {
-    const int t = blockIdx.x;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        double2 a = make_double2(0, 0), b = make_double2(0, 0);
-        double c = 0.0;
-        for (int k = 0; k < nblk; ++k) {
-            const size_t o = ((size_t)t * nblk + k) * n + j;
-            a.x += part_r[o].x;
-            a.y += part_r[o].y;
-            b.x += part_sr[o].x;
-            b.y += part_sr[o].y;
-            c += part_s[o];
-        }
-        const double inv = 1.0 / ns;
-        a.x *= inv; a.y *= inv; b.x *= inv; b.y *= inv; c *= inv;
-        mean_r[(size_t)t * n + j] = a;
-        mean_sr[(size_t)t * n + j] = b;
-        mean_s[(size_t)t * n + j] = c;
-        if (lpl) {
-            const int od = opidx[j], og = opidx[n + j];
-            if (od >= 0) lpl[(size_t)t * nops + od] = site[2 * n + j] * a.x;
-            if (og >= 0) lpl[(size_t)t * nops + og] = 2.0 * site[3 * n + j] * c;
-        }
+// mean_r_j = <r_j> (local sx_j), mean_s_j = <sigma_j>; then <L + L^+> = sqrt(kappa_j) Re mean_r_j
+// (decay), 2 sqrt(gamma_j) mean_s_j (dephasing).  A CTA per 32 sites, a warp each for Re r, Im r and
+// sigma, eight partials loaded ahead of their additions, which keep their order: the kernel was a
+// chain of dependent loads and FP64 additions on one CTA per trajectory (100 trajectories of 160
+// sites, 512 partials: 500 us).
+__global__ void __launch_bounds__(96) site_means_kernel(int n, int nblk, int ns, int nops,
+                                                        const double2* __restrict__ part_r,
+                                                        const double* __restrict__ part_s,
+                                                        const double* __restrict__ site, const int* __restrict__ opidx,
+                                                        double2* __restrict__ mean_r, double* __restrict__ mean_s,
+                                                        double* __restrict__ lpl) {
+    const int t = blockIdx.y, q = threadIdx.x >> 5, j = blockIdx.x * 32 + (threadIdx.x & 31);
+    if (j >= n) return;
+    const size_t o = (size_t)t * nblk * n + j;
+    const double* src = q < 2 ? reinterpret_cast<const double*>(part_r + o) + q : part_s + o;
+    const size_t step = (q < 2 ? 2 : 1) * (size_t)n;
+    double sum = 0.0;
+    int k = 0;
+    for (; k + 8 <= nblk; k += 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = src[(k + u) * step];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) sum += v[u];
+    }
+    for (; k < nblk; ++k) sum += src[k * step];
+    sum *= 1.0 / ns;
+    if (q < 2) reinterpret_cast<double*>(mean_r + (size_t)t * n + j)[q] = sum;
+    else mean_s[(size_t)t * n + j] = sum;
+    if (lpl) {
+        const int od = opidx[j], og = opidx[n + j];
+        if (q == 0 && od >= 0) lpl[(size_t)t * nops + od] = site[2 * n + j] * sum;
+        if (q == 2 && og >= 0) lpl[(size_t)t * nops + og] = 2.0 * site[3 * n + j] * sum;
     }
 }
 
@@ -342,10 +346,9 @@ cudaError_t launch_site_means(const otvmc_ansatz* a, int ntraj, int ns, bool fp3
     ProfScope prof_(OTVMC_K_REDUCE, s);
     const otvmc_model* m = a->model;
     // the per-site partials come from the tensor-core estimators (est_tc_chunks) or the SIMT ones
-    site_means_kernel<<<ntraj, 256, 0, s>>>(a->n, est_tc_ok(a, fp32) ? est_tc_chunks(ns) : est_blocks(a->n, ns), ns,
-                                            m->nops,
-                                            b.part_r, b.part_sr, b.part_s,
-                                            m->site_d, m->opidx_d, b.mean_r, b.mean_sr, b.mean_s, lpl);
+    site_means_kernel<<<dim3((a->n + 31) / 32, ntraj), 96, 0, s>>>(
+        a->n, est_tc_ok(a, fp32) ? est_tc_chunks(ns) : est_blocks(a->n, ns), ns, m->nops, b.part_r, b.part_s, m->site_d,
+        m->opidx_d, b.mean_r, b.mean_s, lpl);
     count_launch();
     return cudaGetLastError();
 }

@@ -3,14 +3,14 @@
 // taken in the same order and precision as est1_jastrow_kernel<true> and
 // observables_kernel<float2, float, .>, so that every result is the same bit for bit.
 //
-// Bound: instruction issue (about 5 and 14 instructions a term).  The kernels they replace were
+// Bound: instruction issue and shared memory.  The kernels they replace were
 // bound by the tables instead: eight samples a CTA read all N^2 entries of three 64-bit tables
 // (0.6 MB at N = 160) from L2, and the observables read one 8-byte table entry from shared memory
 // per term with one CTA of eight warps on an SM.  Here a CTA takes as many samples as its threads
 // hold, records of 16 bytes (converted once per trajectory) arrive in chunks of 16 rows by
 // asynchronous copies one chunk ahead, and a record in registers serves several samples.
-// Estimators of 100 x 4096 samples of 160 sites: 8.7 -> 5.8 ms; observables of 64 x 8192 samples of
-// 100 sites: 11.9 -> 4.6 ms (18 instructions a term, three quarters of the issue slots).
+// Estimators of 100 x 4096 samples of 160 sites: 8.7 -> 4.06 ms; observables of 64 x 8192 samples of
+// 100 sites: 11.9 -> 4.52 ms (16.5 instructions a term, 72 % of the issue slots).
 #include "common.cuh"
 
 namespace otvmc {
@@ -18,6 +18,7 @@ namespace wide {
 
 constexpr int KC = 16;             // rows of a staged chunk
 constexpr int EST_Q = EST_SAMPLES_PER_THREAD;
+constexpr int EST_G = KC / 4;      // groups of eight samples per CTA, each building one group's table
 constexpr int OBS_Q = 4;           // samples of a thread at a time
 constexpr int OBS_VB = 2;          // blocks of 256 threads (in the partials' layout) per CTA
 
@@ -28,95 +29,149 @@ inline size_t r_bytes(int ntraj, int ns, int n) { return ((size_t)ntraj * ns * n
 __device__ __forceinline__ void cp16(void* dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
 }
+__device__ __forceinline__ void cp8(void* dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src));
+}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;"); }
 __device__ __forceinline__ void cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
 // ------------------------------------------------------------------------------- estimators
-// Re and J coupling in FP32, Im in fixed point (units of 2^-48).
-struct alignas(16) EstRec {
-    float re, J;
-    long long im;
-};
-
+// FP32 copies of Re eta and J, a record per (k, j).
 __global__ void __launch_bounds__(256) est_rec_kernel(int n, const long long* __restrict__ Qre,
-                                                      const long long* __restrict__ Qim,
-                                                      const long long* __restrict__ QJ, EstRec* __restrict__ rec) {
+                                                      const long long* __restrict__ QJ, float2* __restrict__ rec) {
     const int t = blockIdx.y, i = blockIdx.x * 256 + threadIdx.x;
     if (i >= n * n) return;
     const size_t o = (size_t)t * n * n + i;
-    rec[o] = EstRec{fx_to_float(Qre[o]), fx_to_float(QJ[i]), Qim[o]};
+    rec[o] = make_float2(fx_to_float(Qre[o]), fx_to_float(QJ[i]));
 }
 
-// Adds a record where the bit is set.  Predicated additions: a conditional statement was compiled to
-// a branch per sample and term, four times the instructions.
-__device__ __forceinline__ void add_if(uint32_t w, uint32_t bit, longlong2 e, uint64_t& af, long long& ai) {
-    asm("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\t"
-        "and.b32 t, %2, %3;\n\t"
-        "setp.ne.u32 p, t, 0;\n\t"
-        "@p add.rn.f32x2 %0, %0, %4;\n\t"
-        "@p add.s64 %1, %1, %5;\n\t}"
-        : "+l"(af), "+l"(ai)
-        : "r"(w), "r"(bit), "l"(e.x), "l"(e.y));
-}
+struct EstSmem {  // byte offsets
+    int rec, ms, offs, sw, total;
+    __host__ __device__ EstSmem(int n, int W, int S) {  // S samples
+        const int nc = (n + KC - 1) / KC;
+        rec = 4 * 16 * n * 8;                 // after the table [4][16][n], later the E_H partials
+        ms = rec + 2 * KC * n * 8;            // records [2][KC][n]
+        offs = ms + S * nc * KC * 4;          // sigma_k = +1 as 1.f or 0.f, [S][nc KC]
+        sw = offs + S * nc * 16;              // table offsets of a chunk's four groups, [S][nc]
+        total = sw + S * W * 8;               // spin words
+    }
+};
 
 // Groups of NT threads, thread j of a group owning site j of the group's eight samples: the block of
 // eight samples is est1_jastrow_kernel's CTA beyond 128 sites, with its partial of the site sums.
-__global__ void __launch_bounds__(1024, 1) est1_wide_kernel(
-    int n, int W, int ns, int nblk, double h, const uint64_t* __restrict__ spins, const EstRec* __restrict__ rec,
-    const long long* __restrict__ base_re, const long long* __restrict__ base_im, const long long* __restrict__ baseJ,
-    float2* __restrict__ r_out, double2* __restrict__ EH_out, double2* __restrict__ part_r,
-    double2* __restrict__ part_sr, double* __restrict__ part_s) {
-    const int NT = ((n + 31) / 32) * 32, G = blockDim.x / NT, t = blockIdx.y;
+// The real and J fields take every k in order, fma(0 or 1, entry, sum); the imaginary field, whole
+// numbers, takes four k at a time from a table of their 16 partial sums, built per chunk and shared
+// by the CTA's samples.  3.5 instructions a term (predicated additions: 10, bound by the half-rate
+// integer pipe).
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) est1_wide_kernel(
+    int n, int W, int ns, int nblk, double h, const uint64_t* __restrict__ spins, const float2* __restrict__ rec,
+    const long long* __restrict__ Qim, const long long* __restrict__ base_re, const long long* __restrict__ base_im,
+    const long long* __restrict__ baseJ, float2* __restrict__ r_out, double2* __restrict__ EH_out,
+    double2* __restrict__ part_r, double2* __restrict__ part_sr, double* __restrict__ part_s) {
+    const int NT = ((n + 31) / 32) * 32, t = blockIdx.y;
+    constexpr int G = EST_G;
     const int g = threadIdx.x / NT, j = threadIdx.x % NT, blk = blockIdx.x * G + g;
     const bool active = j < n && blk < nblk;
+    const int nc = (n + KC - 1) / KC, S = G * EST_Q;
+    const EstSmem lay(n, W, S);
     extern __shared__ __align__(16) unsigned char smraw[];
-    EstRec* tab = reinterpret_cast<EstRec*>(smraw);                    // [2][KC][n]
-    double2* ered = reinterpret_cast<double2*>(tab + 2 * KC * n);      // [G * EST_Q][NT / 32]
-    uint64_t* sw = reinterpret_cast<uint64_t*>(ered + G * EST_Q * (NT / 32));  // [G * EST_Q][W]
-    const int s_first = blockIdx.x * G * EST_Q;
-    const EstRec* rt = rec + (size_t)t * n * n;
+    long long* tab = reinterpret_cast<long long*>(smraw);
+    float2* recs = reinterpret_cast<float2*>(smraw + lay.rec);
+    float* ms = reinterpret_cast<float*>(smraw + lay.ms);
+    int* offs = reinterpret_cast<int*>(smraw + lay.offs);
+    uint64_t* sw = reinterpret_cast<uint64_t*>(smraw + lay.sw);
+    double2* ered = reinterpret_cast<double2*>(smraw);  // [S][NT / 32]
+    const int s_first = blockIdx.x * S;
+    const float2* rt = rec + (size_t)t * n * n;
+    const long long* qt = Qim + (size_t)t * n * n + j;
     auto stage = [&](int c) {
+        float2* dst = recs + (c & 1) * KC * n;
         const int cnt = min(KC, n - c * KC) * n;
-        for (int i = threadIdx.x; i < cnt; i += blockDim.x)
-            cp16(tab + (c & 1) * KC * n + i, rt + (size_t)c * KC * n + i);
+        for (int i = threadIdx.x; i < KC * n; i += blockDim.x) {
+            if (i < cnt) cp8(dst + i, rt + (size_t)c * KC * n + i);
+            else dst[i] = make_float2(0.f, 0.f);
+        }
         cp_commit();
     };
+    long long q4[4] = {0, 0, 0, 0};  // Im of four rows of the next chunk
+    auto fetch = [&](int c) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int k = c * KC + 4 * g + u;
+            q4[u] = k < n ? qt[(size_t)k * n] : 0;
+        }
+    };
+    const bool builds = j < n;
     stage(0);
-    for (int i = threadIdx.x; i < G * EST_Q * W; i += blockDim.x) {
+    if (builds) fetch(0);
+    for (int i = threadIdx.x; i < S * W; i += blockDim.x) {
         const int s = s_first + i / W;
         sw[i] = s < ns ? spins[((size_t)t * ns + s) * W + i % W] : 0ull;
     }
-    uint64_t af[EST_Q];  // FP32 sums of Re eta (low half) and J (high half)
+    __syncthreads();
+    for (int i = threadIdx.x; i < S * nc * KC; i += blockDim.x) {
+        const int s = i / (nc * KC), k = i % (nc * KC);
+        ms[i] = k < n && (sw[s * W + (k >> 6)] >> (k & 63)) & 1ull ? 1.f : 0.f;
+    }
+    for (int i = threadIdx.x; i < S * nc * 4; i += blockDim.x) {
+        const int s = i / (nc * 4), c = i / 4 % nc, q = i & 3;
+        offs[i] = (16 * q + ((int)(sw[s * W + (c >> 2)] >> (KC * (c & 3) + 4 * q)) & 15)) * n * 8;
+    }
+    float ar[EST_Q], aj[EST_Q];
     long long ai[EST_Q];
 #pragma unroll
     for (int q = 0; q < EST_Q; ++q) {
-        af[q] = 0;
+        ar[q] = aj[q] = 0.f;
         ai[q] = 0;
     }
     const uint64_t* sg = sw + g * EST_Q * W;
-    const int nc = (n + KC - 1) / KC;
+    const float* mg = ms + g * EST_Q * nc * KC;
+    const int4* og = reinterpret_cast<const int4*>(offs) + g * EST_Q * nc;
+    const unsigned char* tj = smraw + 8 * j;
     for (int c = 0; c < nc; ++c) {
         cp_wait_all();
-        __syncthreads();  // chunk c is here, and the other buffer has been read
+        __syncthreads();  // the records are here; the table and the other buffer have been read
+        if (builds) {
+            long long* tb = tab + (size_t)16 * g * n + j;
+            const long long s01 = q4[0] + q4[1], s23 = q4[2] + q4[3];
+#pragma unroll
+            for (int p = 0; p < 16; ++p) {
+                const long long lo = (p & 3) == 3 ? s01 : (p & 1) ? q4[0] : (p & 2) ? q4[1] : 0;
+                const long long hi = (p & 12) == 12 ? s23 : (p & 4) ? q4[2] : (p & 8) ? q4[3] : 0;
+                tb[p * n] = lo + hi;
+            }
+            if (c + 1 < nc) fetch(c + 1);
+        }
         if (c + 1 < nc) stage(c + 1);
-        if (active) {
-            const EstRec* tc = tab + (c & 1) * KC * n + j;
-            // 16 bits of each sample, two samples a word; rows beyond n are not staged
-            const uint32_t mask = n - c * KC < KC ? (1u << (n - c * KC)) - 1u : 0xFFFFu;
-            uint32_t w[EST_Q / 2];
+        __syncthreads();
+        if (!active) continue;
+#pragma unroll
+        for (int q = 0; q < EST_Q; ++q) {
+            const int4 o = og[q * nc + c];
+            ai[q] += (*reinterpret_cast<const long long*>(tj + o.x) + *reinterpret_cast<const long long*>(tj + o.y)) +
+                     (*reinterpret_cast<const long long*>(tj + o.z) + *reinterpret_cast<const long long*>(tj + o.w));
+        }
+        const float2* rc = recs + (c & 1) * KC * n + j;
+        const float* mc = mg + c * KC;
+#pragma unroll
+        for (int k4 = 0; k4 < KC; k4 += 4) {
+            float2 e[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) e[u] = rc[(k4 + u) * n];
 #pragma unroll
             for (int q = 0; q < EST_Q; ++q) {
-                const uint32_t x = (uint32_t)(sg[q * W + (c >> 2)] >> (KC * (c & 3))) & mask;
-                w[q / 2] = q & 1 ? w[q / 2] | (x << 16) : x;
-            }
+                const float4 m = *reinterpret_cast<const float4*>(mc + q * nc * KC + k4);
+                const float mv[4] = {m.x, m.y, m.z, m.w};
 #pragma unroll
-            for (int kk = 0; kk < KC; ++kk) {
-                const longlong2 e = *reinterpret_cast<const longlong2*>(tc + kk * n);
-#pragma unroll
-                for (int q = 0; q < EST_Q; ++q) add_if(w[q / 2], 1u << (kk + 16 * (q & 1)), e, af[q], ai[q]);
+                for (int u = 0; u < 4; ++u) {
+                    ar[q] = fmaf(mv[u], e[u].x, ar[q]);
+                    aj[q] = fmaf(mv[u], e[u].y, aj[q]);
+                }
             }
         }
     }
+    __syncthreads();  // the table has been read
     const int lane = threadIdx.x & 31, nw = NT / 32;
     float2 pr = make_float2(0.f, 0.f), psr = make_float2(0.f, 0.f);
     int ps = 0;
@@ -129,9 +184,9 @@ __global__ void __launch_bounds__(1024, 1) est1_wide_kernel(
         float hrx = 0.f, hry = 0.f, fsg = 0.f;
         if (active && s < ns) {
             const bool up = (sg[q * W + (j >> 6)] >> (j & 63)) & 1ull;
-            const float fre = fmaf(2.f, __uint_as_float((uint32_t)af[q]), bre);
+            const float fre = fmaf(2.f, ar[q], bre);
             const long long fim = bim + 2 * ai[q];
-            const float fj = fmaf(2.f, __uint_as_float((uint32_t)(af[q] >> 32)), bj);
+            const float fj = fmaf(2.f, aj[q], bj);
             // log r_j = -2 sigma_j f_j
             const long long lim = up ? -2 * fim : 2 * fim;
             const float e = expf(up ? -2.f * fre : 2.f * fre);
@@ -262,9 +317,9 @@ __global__ void __launch_bounds__(256 * OBS_VB, 2) obs_wide_kernel(int n, int W,
             }
         }
         float2 a2[OBS_Q], b2[OBS_Q];
-        uint32_t flip = 0;  // bit i: s_j = -1 in sample i
+        float sj[OBS_Q];  // s_j
 #pragma unroll
-        for (int i = 0; i < OBS_Q; ++i) a2[i] = b2[i] = make_float2(0.f, 0.f);
+        for (int i = 0; i < OBS_Q; ++i) a2[i] = b2[i] = make_float2(sj[i] = 0.f, 0.f);
         for (int c = 0; c < nc; ++c) {
             cp_wait_all();
             __syncthreads();  // chunk c (and the samples) are here, the other buffer has been read
@@ -272,24 +327,16 @@ __global__ void __launch_bounds__(256 * OBS_VB, 2) obs_wide_kernel(int n, int W,
             if (!active) continue;
             if (c == 0)
 #pragma unroll
-                for (int i = 0; i < OBS_Q; ++i) flip |= (rg[i * n + j].z < 0.f ? 1u : 0u) << i;
-            // bit kk of sample i's half word: s_j = s_k for k = 16 c + kk
-            uint32_t x[OBS_Q / 2];
-#pragma unroll
-            for (int i = 0; i < OBS_Q; ++i) {
-                uint32_t y = (uint32_t)(sg[i * W + (c >> 2)] >> (KC * (c & 3)));
-                if ((flip >> i) & 1u) y = ~y;
-                x[i / 2] = i & 1 ? x[i / 2] | (y << 16) : y & 0xFFFFu;
-            }
+                for (int i = 0; i < OBS_Q; ++i) sj[i] = rg[i * n + j].z;
             const float4* tc = tab + (c & 1) * KC * n + j;
             const float4* rc = rg + c * KC;
             auto term = [&](int kk) {
                 const float4 E = tc[kk * n];
 #pragma unroll
                 for (int i = 0; i < OBS_Q; ++i) {
-                    const bool same = x[i / 2] & (1u << (kk + 16 * (i & 1)));
-                    const float2 e = make_float2(same ? E.x : E.z, same ? E.y : E.w);
                     const float4 rk = rc[i * n + kk];
+                    const bool same = rk.z == sj[i];
+                    const float2 e = make_float2(same ? E.x : E.z, same ? E.y : E.w);
                     const float2 p = cmul_fma(rk.x, rk.y, e);
                     a2[i].x += p.x;
                     a2[i].y += p.y;
@@ -312,18 +359,17 @@ __global__ void __launch_bounds__(256 * OBS_VB, 2) obs_wide_kernel(int n, int W,
             int S = 0;
             for (int ww = 0; ww < W; ++ww) S += 2 * __popcll(sg[i * W + ww]);
             S -= n;
-            const int sj = (flip >> i) & 1u ? -1 : 1;
             const float4 rv = rg[i * n + j];
             const float2 rj = make_float2(rv.x, rv.y);
             float2 a = a2[i], bb = b2[i];
             // the diagonal's term r_j (and sigma_j r_j) taken out again
             a.x -= rj.x;
             a.y -= rj.y;
-            bb.x -= (float)sj * rj.x;
-            bb.y -= (float)sj * rj.y;
+            bb.x -= sj[i] * rj.x;
+            bb.y -= sj[i] * rj.y;
             const float rax = cmul_fma(rj.x, rj.y, a).x;
             const float2 rb = cmul_fma(rj.x, rj.y, bb);
-            const float fs = (float)sj, fS = (float)(S - sj);
+            const float fs = sj[i], fS = (float)S - fs;
             acc[0] += rj.x;
             acc[1] += fs * rj.y;
             acc[2] += fs;
@@ -353,7 +399,7 @@ __global__ void __launch_bounds__(256 * OBS_VB, 2) obs_wide_kernel(int n, int W,
 bool est_wide_ok(const otvmc_ansatz* a, bool fp32, int ntraj, int ns) {
     if (!fp32 || a->kind != OTVMC_JASTROW || a->n <= ETC_MAX_N) return false;
     const size_t n = a->n;
-    return wide::r_bytes(ntraj, ns, a->n) + (size_t)ntraj * n * n * 16 <= (size_t)ntraj * ns * n * 16;
+    return wide::r_bytes(ntraj, ns, a->n) + (size_t)ntraj * n * n * 8 <= (size_t)ntraj * ns * n * 16;
 }
 
 cudaError_t launch_est1_wide(const otvmc_ansatz* a, const uint64_t* spins, int ntraj, int ns, const EvalBufs& b,
@@ -362,16 +408,16 @@ cudaError_t launch_est1_wide(const otvmc_ansatz* a, const uint64_t* spins, int n
     ProfScope prof_(OTVMC_K_EST1, s);
     const int n = a->n, W = (n + 63) / 64, NT = ((n + 31) / 32) * 32, nblk = est_blocks(n, ns);
     const otvmc_model* m = a->model;
-    EstRec* rec = reinterpret_cast<EstRec*>(reinterpret_cast<char*>(b.r) + r_bytes(ntraj, ns, n));
-    est_rec_kernel<<<dim3((n * n + 255) / 256, ntraj), 256, 0, s>>>(n, b.Qre, b.Qim, m->QJ_d, rec);
+    float2* rec = reinterpret_cast<float2*>(reinterpret_cast<char*>(b.r) + r_bytes(ntraj, ns, n));
+    est_rec_kernel<<<dim3((n * n + 255) / 256, ntraj), 256, 0, s>>>(n, b.Qre, m->QJ_d, rec);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    const int G = 1024 / NT < nblk ? 1024 / NT : nblk;
-    const size_t smem = (size_t)2 * KC * n * 16 + (size_t)G * EST_Q * (NT / 32 * 16 + W * 8);
-    e = cudaFuncSetAttribute(est1_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    auto kern = NT <= 160 ? est1_wide_kernel<640> : NT <= 192 ? est1_wide_kernel<768> : est1_wide_kernel<896>;
+    const size_t smem = EstSmem(n, W, EST_G * EST_Q).total;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    est1_wide_kernel<<<dim3((nblk + G - 1) / G, ntraj), G * NT, smem, s>>>(
-        n, W, ns, nblk, m->h, spins, rec, b.base_re, b.base_im, m->baseJ_d, reinterpret_cast<float2*>(b.r), b.EH,
+    kern<<<dim3((nblk + EST_G - 1) / EST_G, ntraj), EST_G * NT, smem, s>>>(
+        n, W, ns, nblk, m->h, spins, rec, b.Qim, b.base_re, b.base_im, m->baseJ_d, reinterpret_cast<float2*>(b.r), b.EH,
         b.part_r, b.part_sr, b.part_s);
     count_launch(2);
     return cudaGetLastError();
