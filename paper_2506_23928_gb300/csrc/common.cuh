@@ -83,4 +83,18 @@ __device__ __forceinline__ double2 cexp_prec(double re, double im, bool fp32) {
     return make_double2((double)(e * c), (double)(e * s));
 }
 
+// The nine moments of 256 threads' rows red[256][9] added up by `warps` warps of which this is `warp`, a
+// moment per warp and turn (a thread per moment took a chain of 256 FP64 additions).
+__device__ __forceinline__ void obs_block_sum(const double* red, int warp, int warps, double* out) {
+    const int lane = threadIdx.x & 31;
+    for (int i = warp; i < 9; i += warps) {
+        double s = 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += red[(lane + 32 * u) * 9 + i];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if (lane == 0) out[i] = s;
+    }
+}
+
 }  // namespace otvmc

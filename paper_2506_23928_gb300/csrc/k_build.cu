@@ -180,12 +180,22 @@ __device__ __forceinline__ uint4 e4m3_pm1x16(uint32_t e) {
 
 // E4M3 code of an integer |d| <= 8, from the format's definition: sign bit, exponent biased by
 // 7 (bits 3..6), three fraction bits; d = 2^e (1 + f / 8).
-__device__ __forceinline__ uint32_t e4m3_small_int(int d) {
-    if (d == 0) return 0u;
-    const uint32_t sg = d < 0 ? 0x80u : 0u;
-    const int a = d < 0 ? -d : d;
-    const int e = 31 - __clz(a);
-    return sg | ((uint32_t)(e + 7) << 3) | (uint32_t)((a << (3 - e)) - 8);
+__host__ __device__ constexpr uint32_t e4m3_small_int(int d) {
+    const int a = d < 0 ? -d : d, e = a >= 8 ? 3 : a >= 4 ? 2 : a >= 2 ? 1 : 0;
+    return d == 0 ? 0u : (d < 0 ? 0x80u : 0u) | ((uint32_t)(e + 7) << 3) | (uint32_t)((a << (3 - e)) - 8);
+}
+// The codes of d, d + 1, d + 2 and d + 3, one per byte.
+__host__ __device__ constexpr uint32_t e4m3_codes4(int d) {
+    return e4m3_small_int(d) | e4m3_small_int(d + 1) << 8 | e4m3_small_int(d + 2) << 16 | e4m3_small_int(d + 3) << 24;
+}
+// Four codes of u - 8, u = the four nibbles of v (0 .. 15): byte permutes of the sixteen codes.
+__device__ __forceinline__ uint32_t e4m3_nibbles(uint32_t v) {
+    const uint32_t sel = v & 0x7777u, x = (v >> 3) & 0x1111u;
+    const uint32_t y = (x & 0x0011u) | ((x & 0x1100u) << 8);                 // bits 0, 4, 16, 20
+    const uint32_t up = ((y & 0x00010001u) | ((y & 0x00100010u) << 4)) * 255u;  // a byte mask of u >= 8
+    const uint32_t neg = __byte_perm(e4m3_codes4(-8), e4m3_codes4(-4), sel);
+    const uint32_t pos = __byte_perm(e4m3_codes4(0), e4m3_codes4(4), sel);
+    return (pos & up) | (neg & ~up);
 }
 
 __global__ void __launch_bounds__(OB_THREADS) obuild_f8_jastrow_kernel(int n, int W, int P, int rows, int ns,
@@ -233,26 +243,33 @@ __global__ void __launch_bounds__(OB_THREADS) obuild_f8_jastrow_kernel(int n, in
         *reinterpret_cast<uint4*>(base + (size_t)k * pitch) = make_uint4(v.x & vm[0], v.y & vm[1], v.z & vm[2],
                                                                          v.w & vm[3]);
     }
-    if (qv == nullptr || blockIdx.z != gridDim.z - 1) return;
-    // extra rows P .. P + 32: the balanced base-16 digits d_p in [-8, 7] of q (real part, then
-    // imaginary part; q = sum_p d_p 16^p), then ones; 0 for the samples from ns on
+    if (qv == nullptr) return;
+    // extra rows P .. P + 32, split over gridDim.z like the parameters: the balanced base-16 digits
+    // d_p in [-8, 7] of q (real part, then imaginary part; q = sum_p d_p 16^p), then ones; 0 for the
+    // samples from ns on.  d_p + 8 is the p-th nibble of q + 0x88...8 (modulo 2^64).
+    const int e0 = 33 * (int)blockIdx.z / (int)gridDim.z, e1 = 33 * ((int)blockIdx.z + 1) / (int)gridDim.z;
 #pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-        long long r[OB_SPT];
+    for (int h8 = 0; h8 < 4; ++h8) {  // real and imaginary part, low and high half of the digits
+        const int r0 = max(e0, 8 * h8), r1 = min(e1, 8 * h8 + 8);
+        if (r0 >= r1) continue;
+        uint32_t r[OB_SPT];
 #pragma unroll
-        for (int q = 0; q < OB_SPT; ++q) r[q] = (x0 + q < ns) ? qv[((size_t)t * ns + x0 + q) * 2 + h] : 0ll;
+        for (int q = 0; q < OB_SPT; ++q) {
+            const long long v = (x0 + q < ns) ? qv[((size_t)t * ns + x0 + q) * 2 + (h8 >> 1)] : 0ll;
+            r[q] = (uint32_t)(((unsigned long long)v + 0x8888888888888888ull) >> (32 * (h8 & 1)));
+        }
 #pragma unroll 1
-        for (int p = 0; p < 16; ++p) {
-            uint32_t w[4] = {0u, 0u, 0u, 0u};
+        for (int e = r0; e < r1; ++e) {
+            const int sh = 4 * (e & 7);
+            uint32_t w[4];
 #pragma unroll
-            for (int q = 0; q < OB_SPT; ++q) {
-                const int d = (int)((r[q] & 0xF) ^ 0x8) - 0x8;
-                r[q] = (r[q] - d) >> 4;  // exact: r - d is a multiple of 16
-                w[q >> 2] |= e4m3_small_int(d) << (8 * (q & 3));
-            }
-            *reinterpret_cast<uint4*>(base + (size_t)(P + 16 * h + p) * pitch) = make_uint4(w[0], w[1], w[2], w[3]);
+            for (int q = 0; q < 4; ++q)
+                w[q] = e4m3_nibbles(((r[4 * q] >> sh) & 0xFu) | (((r[4 * q + 1] >> sh) & 0xFu) << 4) |
+                                    (((r[4 * q + 2] >> sh) & 0xFu) << 8) | (((r[4 * q + 3] >> sh) & 0xFu) << 12));
+            *reinterpret_cast<uint4*>(base + (size_t)(P + e) * pitch) = make_uint4(w[0], w[1], w[2], w[3]);
         }
     }
+    if (e1 != 33) return;
     *reinterpret_cast<uint4*>(base + (size_t)(P + 32) * pitch) =
         make_uint4(0x38383838u & vm[0], 0x38383838u & vm[1], 0x38383838u & vm[2], 0x38383838u & vm[3]);
 }
@@ -265,13 +282,15 @@ cudaError_t launch_obuild_f8_jastrow(const otvmc_ansatz* a, const uint64_t* spin
     const int rows = qv != nullptr ? P + D_XROWS : P;
     const int per_block = OB_THREADS * OB_SPT;
     const int gx = (pitch + per_block - 1) / per_block;
-    // parameter ranges: about eight blocks per SM over the batch, each range >= 64 parameters
+    // ranges of parameters and digit rows: about eight blocks per SM over the batch, each range >= 64
+    // parameters, but up to four blocks for the digit rows alone (16 trajectories of 8 spins, 1024
+    // samples: 38 -> 8 us, where one block a trajectory wrote 69 rows)
     int dev = 0, sms = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         sms <= 0)
         sms = 152;
     int kz = (8 * sms + gx * ntraj - 1) / (gx * ntraj);
-    kz = max(1, min(kz, P / 64));
+    kz = max(1, min(kz, max(P / 64, qv != nullptr ? 4 : 1)));
     dim3 grid(gx, ntraj, kz);
     const size_t smem = (size_t)n * OB_THREADS * sizeof(uint16_t);
     if (smem > 48 * 1024) {

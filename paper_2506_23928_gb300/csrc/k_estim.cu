@@ -636,8 +636,16 @@ __global__ void vquant_kernel(int ns, int vblk, const double2* __restrict__ v, c
         lr += a;
         li += b;
     }
-    atomicAdd(&acc[0], (unsigned long long)lr);
-    atomicAdd(&acc[1], (unsigned long long)li);
+    // (a shared-memory atomic per warp: one per thread queued up for 15 us)
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        lr += __shfl_xor_sync(0xffffffffu, lr, off);
+        li += __shfl_xor_sync(0xffffffffu, li, off);
+    }
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&acc[0], (unsigned long long)lr);
+        atomicAdd(&acc[1], (unsigned long long)li);
+    }
     __syncthreads();
     if (threadIdx.x == 0) {
         qsum[2 * t] = (long long)acc[0];
@@ -722,24 +730,38 @@ __global__ void __launch_bounds__(256) observables_kernel(int n, int W, int ns, 
     R acc[9];  // per-thread sums over its spt samples (FP32 on the MIXED path), then FP64
 #pragma unroll
     for (int i = 0; i < 9; ++i) acc[i] = (R)0;
+    // the next sample's ratio (and its spins, where they are one word) are loaded a sample ahead
+    const auto sample = [&](int q) { return blk * SB + g + q * SPP; };
+    const auto used = [&](int q) { return active && q < spt && sample(q) < ns; };
+    R2 r_next = {0, 0};
+    uint64_t w_next = 0;
+    if (used(0)) {
+        r_next = r[((size_t)t * ns + sample(0)) * n + j];
+        w_next = spins[((size_t)t * ns + sample(0)) * W];
+    }
     for (int q = 0; q < spt; ++q) {
-        const int s = blk * SB + g + q * SPP;
+        const int s = sample(q);
         __syncthreads();
-        if (active && s < ns) rs[g * NT + j] = r[((size_t)t * ns + s) * n + j];
+        if (active) rs[g * NT + j] = r_next;
         __syncthreads();
-        if (!(active && s < ns)) continue;
+        const uint64_t w0 = w_next;
+        if (used(q + 1)) {
+            r_next = r[((size_t)t * ns + sample(q + 1)) * n + j];
+            w_next = spins[((size_t)t * ns + sample(q + 1)) * W];
+        }
+        if (!used(q)) continue;
         const uint64_t* w = spins + ((size_t)t * ns + s) * W;
-        int S = 0;
-        for (int ww = 0; ww < W; ++ww) S += 2 * __popcll(w[ww]);
+        int S = 2 * __popcll(w0);
+        for (int ww = 1; ww < W; ++ww) S += 2 * __popcll(w[ww]);
         S -= n;
-        const uint64_t sjb = (w[j >> 6] >> (j & 63)) & 1ull;
+        const uint64_t sjb = ((j < 64 ? w0 : w[j >> 6]) >> (j & 63)) & 1ull;
         const int sj = sjb ? 1 : -1;
         R2 a2 = {0, 0}, b2 = {0, 0};
         const R2* rr = rs + g * NT;
         // all k, the diagonal included (E^{+}_jj = 1), whose term r_j (and sigma_j r_j) is
         // removed after the loop
         for (int k0 = 0; k0 < n; k0 += 64) {
-            uint64_t word = w[k0 >> 6];
+            uint64_t word = k0 == 0 ? w0 : w[k0 >> 6];
             const int kend = min(64, n - k0);
 #pragma unroll 4
             for (int kk = 0; kk < kend; ++kk, word >>= 1) {
@@ -782,11 +804,7 @@ __global__ void __launch_bounds__(256) observables_kernel(int n, int W, int ns, 
 #pragma unroll
     for (int i = 0; i < 9; ++i) red[threadIdx.x * 9 + i] = (double)acc[i];
     __syncthreads();
-    if (threadIdx.x < 9) {
-        double sum = 0.0;
-        for (int k = 0; k < 256; ++k) sum += red[k * 9 + threadIdx.x];
-        part_obs[((size_t)t * gridDim.x + blk) * 9 + threadIdx.x] = sum;
-    }
+    obs_block_sum(red, threadIdx.x >> 5, 8, part_obs + ((size_t)t * gridDim.x + blk) * 9);
 }
 
 __global__ void obs_final_kernel(int n, int ns, int nblk, const double* __restrict__ part_obs,

@@ -385,13 +385,7 @@ __global__ void __launch_bounds__(256 * OBS_VB, 2) obs_wide_kernel(int n, int W,
 #pragma unroll
     for (int i = 0; i < 9; ++i) red[threadIdx.x * 9 + i] = (double)acc[i];
     __syncthreads();
-    if (lt < 9 && blk < nblk) {
-        // (threads beyond the last group hold zeros)
-        double sum = 0.0;
-        const int cnt = SPP * NT;
-        for (int k = 0; k < cnt; ++k) sum += red[(vb * 256 + k) * 9 + lt];
-        b.part[((size_t)t * nblk + blk) * 9 + lt] = sum;
-    }
+    if (blk < nblk) obs_block_sum(red + vb * 256 * 9, lt >> 5, 8, b.part + ((size_t)t * nblk + blk) * 9);
 }
 
 }  // namespace wide
