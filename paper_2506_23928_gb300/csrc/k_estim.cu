@@ -667,28 +667,36 @@ cudaError_t launch_vquant(int ntraj, int ns, const double2* v, const EvalBufs& b
 // ---------------------------------------------------------------------- observables
 // Epm[t][0][j][k] = exp(4 eta_jk), Epm[t][1][j][k] = exp(-4 eta_jk): the two-flip ratio is
 // r_jk = r_j r_k exp(4 sigma_j sigma_k eta_jk).
-__global__ void obs_prep_kernel(const double2* __restrict__ theta, int P, int n, double2* __restrict__ Epm) {
-    const int t = blockIdx.x;
-    const double2* th = theta + (size_t)t * P;
-    double2* E = Epm + (size_t)t * 2 * n * n;
-    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
-        const int j = idx / n, k = idx - j * n;
-        double2 p = make_double2(1.0, 0.0), q = make_double2(1.0, 0.0);
-        if (j != k) {
-            const double2 e = th[n + pair_idx(min(j, k), max(j, k), n)];
-            p = cexp_prec(4.0 * e.x, 4.0 * e.y, false);
-            q = cexp_prec(-4.0 * e.x, -4.0 * e.y, false);
-        }
-        E[idx] = p;
-        E[n * n + idx] = q;
-    }
+//
+// A thread per pair j < k (rows j and n - 1 - j together hold n - 1 of them) computes one sine and
+// cosine and both exponentials for the four entries, over as many CTAs as that takes; a CTA per
+// trajectory computed each entry by itself (64 trajectories of 64 sites: 106 -> 12 us).
+__global__ void __launch_bounds__(128) obs_prep_kernel(const double2* __restrict__ theta, int P, int n,
+                                                       double2* __restrict__ Epm) {
+    const int t = blockIdx.y, i = blockIdx.x * 128 + threadIdx.x;
+    const double2* th = theta + (size_t)t * P + n;
+    double2 *Ep = Epm + (size_t)t * 2 * n * n, *Em = Ep + n * n;
+    if (i < n) Ep[i * n + i] = Em[i * n + i] = make_double2(1.0, 0.0);
+    if (n < 2) return;
+    const int row = i / (n - 1), m = i % (n - 1);
+    if (row >= (n + 1) / 2) return;
+    const bool first = m < n - 1 - row;
+    const int j = first ? row : n - 1 - row, k = j + 1 + (first ? m : m - (n - 1 - row));
+    if (k >= n) return;
+    const double2 e = th[pair_idx(j, k, n)];
+    double s, c;
+    sincos(4.0 * e.y, &s, &c);
+    const double ep = exp(4.0 * e.x), em = exp(-4.0 * e.x);
+    Ep[j * n + k] = Ep[k * n + j] = make_double2(ep * c, ep * s);
+    Em[j * n + k] = Em[k * n + j] = make_double2(em * c, em * -s);
 }
 
 cudaError_t launch_obs_prep(const otvmc_ansatz* a, const double2* theta, int ntraj, bool fp32, const EvalBufs& b,
                             cudaStream_t s) {
     ProfScope prof_(OTVMC_K_OBS, s);
     if (obs_wide_ok(a, fp32)) return launch_obs_prep_wide(a, theta, ntraj, b, s);
-    obs_prep_kernel<<<ntraj, 256, 0, s>>>(theta, (int)a->P, a->n, b.Epm);
+    const int n = a->n, pairs = (n + 1) / 2 * (n - 1), items = pairs > n ? pairs : n;
+    obs_prep_kernel<<<dim3((items + 127) / 128, ntraj), 128, 0, s>>>(theta, (int)a->P, n, b.Epm);
     count_launch();
     return cudaGetLastError();
 }

@@ -19,7 +19,11 @@
 // an N x (M+1) product over the samples.  The column means obar are the same product with
 // z = 1 and t unconjugated.  The real embedding written for the Cholesky is the one of
 // k_rbm.cu: rows x and ns + x, [[Re T_c, -Im T_c], [Im T_c, Re T_c]], upper triangle.
+#include <cooperative_groups.h>
+
 #include "common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace otvmc {
 namespace rbmf {
@@ -406,6 +410,8 @@ __global__ void __launch_bounds__(256) tanh_fx_kernel(int n, int M, int W, int P
 }
 
 constexpr int XD = 32;  // samples per chunk of the column sums
+constexpr int CS_MAX = 8;      // CTAs that may share the samples of a column block
+constexpr int CS_SUMS = 18;    // 64-bit sums of a thread
 
 // Column sums over the samples, for columns c = 0..M (c = M stands for the constant 1):
 //     Wsum[t][i][c] = sum_x s_i(x) f_c(x) z(x),   csum[t][c] = sum_x f_c(x) z(x),
@@ -415,14 +421,22 @@ constexpr int XD = 32;  // samples per chunk of the column sums
 // f z in FP64, then in fixed point with one scale per CTA from the bound fmax[t] zmax; per site
 // the sum is taken as (sum over all samples) - 2 (sum over the samples where s_i = -1), exactly:
 // the lanes of a warp share sample and site, so the test does not diverge.
+//
+// Where a batch has fewer CTAs than the SMs hold, a cluster of up to eight takes the chunks of samples
+// in turn and its first CTA adds the whole numbers up through distributed shared memory: one CTA
+// a column block walked through all samples, 80 CTAs of 8 warps for 16 trajectories of 128 units (2048
+// samples: 557 -> 244 us).
 __global__ void __launch_bounds__(256) colsum_fx_kernel(int n, int M, int W, int ns, int conj,
                                                         const uint64_t* __restrict__ spins,
                                                         const double2* __restrict__ Td,
                                                         const unsigned long long* __restrict__ fmax_bits,
                                                         const double2* __restrict__ zr, double2* __restrict__ Wsum,
                                                         double2* __restrict__ csum) {
-    const int t = blockIdx.z, ib = blockIdx.y, c0 = blockIdx.x * 32;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), cn = (int)cl.num_blocks();
+    const int t = blockIdx.z, ib = blockIdx.y, c0 = blockIdx.x / cn * 32;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    extern __shared__ long long cs_sums[];  // [CS_SUMS][256] in a cluster of more than one
     __shared__ ll2 fz[XD][33];
     __shared__ uint64_t sb[XD];
     __shared__ double2 zs[XD];
@@ -446,7 +460,7 @@ __global__ void __launch_bounds__(256) colsum_fx_kernel(int n, int M, int W, int
     long long tx = 0, ty = 0, dx[8], dy[8];
 #pragma unroll
     for (int r = 0; r < 8; ++r) dx[r] = dy[r] = 0;
-    for (int x0 = 0; x0 < ns; x0 += XD) {
+    for (int x0 = rank * XD; x0 < ns; x0 += cn * XD) {
         __syncthreads();
         if (tid < XD) {
             const int x = x0 + tid;
@@ -468,7 +482,7 @@ __global__ void __launch_bounds__(256) colsum_fx_kernel(int n, int M, int W, int
                 f = cc < M ? Tt[(size_t)cc * ns + x] : make_double2(1.0, 0.0);
                 if (conj) f.y = -f.y;
             }
-            const double2 w = cmul(f, zs[xs]);
+            const double2 w = zt ? cmul(f, zs[xs]) : f;
             fz[xs][l] = ll2{fxq(w.x, sc), fxq(w.y, sc)};
         }
         __syncthreads();
@@ -486,6 +500,31 @@ __global__ void __launch_bounds__(256) colsum_fx_kernel(int n, int M, int W, int
                 }
         }
     }
+    if (cn > 1) {
+        if (rank > 0) {
+            cs_sums[tid] = tx;
+            cs_sums[256 + tid] = ty;
+#pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                cs_sums[(2 + r) * 256 + tid] = dx[r];
+                cs_sums[(10 + r) * 256 + tid] = dy[r];
+            }
+        }
+        cl.sync();
+        if (rank == 0)
+            for (int o = 1; o < cn; ++o) {
+                const long long* p = cl.map_shared_rank(cs_sums, o) + tid;
+                tx += p[0];
+                ty += p[256];
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    dx[r] += p[(2 + r) * 256];
+                    dy[r] += p[(10 + r) * 256];
+                }
+            }
+        cl.sync();  // the others' shared memory has been read
+        if (rank > 0) return;
+    }
     if (c > M) return;
     const double inv = 1.0 / sc;
 #pragma unroll
@@ -496,6 +535,32 @@ __global__ void __launch_bounds__(256) colsum_fx_kernel(int n, int M, int W, int
                 make_double2((double)(tx - 2 * dx[r]) * inv, (double)(ty - 2 * dy[r]) * inv);
     }
     if (ib == 0 && warp == 0) csum[(size_t)t * (M + 1) + c] = make_double2((double)tx * inv, (double)ty * inv);
+}
+
+static cudaError_t launch_colsum_fx(int T, int n, int M, int W, int ns, int conj, const uint64_t* spins,
+                                    const double2* Td, const unsigned long long* fmax, const double2* zr,
+                                    double2* Wsum, double2* csum, cudaStream_t s) {
+    const int cols = (M + 1 + 31) / 32;
+    // about four CTAs per SM, each with at least two chunks
+    int cn = CS_MAX;
+    while (cn > 1 && ((long long)cols * W * T * cn > 5 * 152 || ns < 2 * XD * cn)) cn /= 2;
+    const size_t smem = cn > 1 ? CS_SUMS * 256 * sizeof(long long) : 0;
+    cudaError_t e = cudaFuncSetAttribute(colsum_fx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         CS_SUMS * 256 * (int)sizeof(long long));
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(cols * cn), (unsigned)W, (unsigned)T);
+    cfg.blockDim = dim3(256);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)cn;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, colsum_fx_kernel, n, M, W, ns, conj, spins, Td, fmax, zr, Wsum, csum);
 }
 
 // r(x) = v_c(x) - eps z(x) - sum_k (O_k(x) - obar_k) y_k for AS samples per CTA, thread = hidden
@@ -659,8 +724,8 @@ cudaError_t launch_rbm_tanh_obar(const otvmc_ansatz* a, const double2* theta, co
     wquant_kernel<<<T, 256, 0, s>>>(n, M, P, theta, wt.q, wt.qs, wt.scale);
     tanh_fx_kernel<<<dim3((ns + AS - 1) / AS, T), hid_threads(M), 0, s>>>(n, M, W, P, ns, theta, spins, wt.q, wt.qs,
                                                                           wt.scale, Td, Tf, fmax);
-    colsum_fx_kernel<<<dim3((M + 1 + 31) / 32, W, T), 256, 0, s>>>(n, M, W, ns, 0, spins, Td, fmax, nullptr, Wsum,
-                                                                   csum);
+    e = launch_colsum_fx(T, n, M, W, ns, 0, spins, Td, fmax, nullptr, Wsum, csum, s);
+    if (e != cudaSuccess) return e;
     finish_kernel<<<dim3((P + 255) / 256, T), 256, 0, s>>>(n, M, P, ns, 0, Wsum, csum, nullptr, obar);
     count_launch(4);
     return cudaGetLastError();
@@ -695,12 +760,12 @@ cudaError_t launch_rbm_refine_push(const otvmc_ansatz* a, int T, int ns, double 
     double2* csum = (double2*)take((size_t)T * (M + 1) * 16);
     take((size_t)T * 2 * P * 16);
     const FxTab yt = take_fxtab(take, n, M, T);
-    const dim3 cs_grid((M + 1 + 31) / 32, W, T);
     for (int it = 0; it <= iters; ++it) {
         double2* out = it == iters ? delta : y;
         {
             ProfScope prof_(OTVMC_K_D, s);
-            colsum_fx_kernel<<<cs_grid, 256, 0, s>>>(n, M, W, ns, 1, spins, Td, fmax, z, Wsum, csum);
+            const cudaError_t ec = launch_colsum_fx(T, n, M, W, ns, 1, spins, Td, fmax, z, Wsum, csum, s);
+            if (ec != cudaSuccess) return ec;
             finish_kernel<<<dim3((P + 255) / 256, T), 256, 0, s>>>(n, M, P, ns, 1, Wsum, csum, obar, out);
             count_launch(2);
         }
@@ -740,7 +805,6 @@ cudaError_t launch_rbm_refine_S(const otvmc_ansatz* a, int T, int ns, double eps
     double2* csum = (double2*)take((size_t)T * (M + 1) * 16);
     double2* re = (double2*)take((size_t)T * 2 * P * 16);
     const FxTab dt = take_fxtab(take, n, M, T);
-    const dim3 cs_grid((M + 1 + 31) / 32, W, T);
     const dim3 pg((P + 255) / 256, T);
     for (int it = 0; it <= iters; ++it) {
         unembed_kernel<<<pg, 256, 0, s>>>(P, xe, delta);
@@ -752,7 +816,8 @@ cudaError_t launch_rbm_refine_S(const otvmc_ansatz* a, int T, int ns, double eps
             wquant_kernel<<<T, 256, 0, s>>>(n, M, P, delta, dt.q, dt.qs, dt.scale);
             resid_fx_kernel<<<dim3((ns + AS - 1) / AS, T), hid_threads(M), 0, s>>>(
                 n, M, W, P, ns, 0.0, spins, Td, obar, delta, dt.q, dt.qs, dt.scale, vemb, vemb, w);
-            colsum_fx_kernel<<<cs_grid, 256, 0, s>>>(n, M, W, ns, 1, spins, Td, fmax, w, Wsum, csum);
+            const cudaError_t ec = launch_colsum_fx(T, n, M, W, ns, 1, spins, Td, fmax, w, Wsum, csum, s);
+            if (ec != cudaSuccess) return ec;
             finish_kernel<<<pg, 256, 0, s>>>(n, M, P, ns, 1, Wsum, csum, obar, g);
             sres_kernel<<<pg, 256, 0, s>>>(P, eps, g, delta, re);
             count_launch(5);
