@@ -490,7 +490,12 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
         }
         if (rank == 0) {
             double rmax = 0.0;
-            for (int i = tid; i < P; i += THREADS) rmax = fmax(rmax, fmax(fabs(__ldcg(gr + i)), fabs(__ldcg(gr + P + i))));
+            // (NaN counts as infinity in block_max; fmax alone would drop it, and a right-hand side of NaN and
+            // zeros would read as zero)
+            for (int i = tid; i < P; i += THREADS) {
+                const double ra = __ldcg(gr + i), rb = __ldcg(gr + P + i);
+                rmax = isfinite(ra) && isfinite(rb) ? fmax(rmax, fmax(fabs(ra), fabs(rb))) : INFINITY;
+            }
             rmax = block_max(rmax, sm.red[0]);
             int stop = 0;  // 1: converged, 2: left to FP64
             if (rmax == 0.0) {
@@ -512,7 +517,6 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
                     const double ds = (double)dsc[i];
                     const double da = (double)y[i] * down, db = (double)y[PY + i] * down;
                     const double xa = __ldcg(gx + i) + da * ds, xb = __ldcg(gx + P + i) + db * ds;
-                    // (NaN counts as infinity in block_max; fmax alone would drop it)
                     ndx = isfinite(da) && isfinite(db) ? fmax(ndx, fmax(fabs(da), fabs(db))) : INFINITY;
                     nx = fmax(nx, fmax(fabs(xa), fabs(xb)) / ds);
                     gx[i] = xa;
@@ -522,7 +526,7 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
                 nx = block_max(nx, sm.red[1]);
                 // rate of the refinement from the last two corrections: what is left after this one is
                 // about rate * ndx.  Corrections at the rounding of x itself cannot shrink further.
-                if (!(ndx < 1e300) || (it > 0 && ndx > 0.25 * prev && ndx > 1e-15 * nx)) {
+                if (!(ndx < 1e300) || !(nx < 1e300) || (it > 0 && ndx > 0.25 * prev && ndx > 1e-15 * nx)) {
                     stop = 2;
                 } else if (it > 0 && (ndx * fmax(ndx / prev, 0x1.0p-22) <= 0x1.0p-54 * nx || ndx <= 1e-15 * nx)) {
                     stop = 1;
