@@ -10,7 +10,8 @@
 //      operands staged by asynchronous copies); one warp of CTA 0 factors and inverts the
 //      diagonal tile (factor32); the CTAs multiply their rows of C by the inverse.
 //   3. r = D - A x (rows over the warps of the cluster), dx from the FP32 factor (CTA 0), x += dx in
-//      FP64, until the next correction, foretold from the last two, is below 2^-54 of x.  The
+//      FP64, until the next correction, foretold from the last two, is below 2^-54 of x, for the real
+//      and the imaginary system separately (a part 1e-8 of the other was left at 3e-11 of itself).  The
 //      residual is taken from whole numbers: d S d and x / d as 63-bit fixed point in three signed
 //      digits of 21 bits, the six leading digit products summed exactly in 64-bit integers.  Its
 //      error is about 2^-61 |x|, below what an FP64 dot product leaves (2^-53 |S| |x|), so that the
@@ -59,7 +60,7 @@ struct alignas(16) Smem {  // its size a multiple of 16: float4 vectors follow i
     float X[TB][TB + 4];
     float scr[4 * TB];
     float t[2][TB];
-    double red[2][WARPS];
+    uint32_t red[2][WARPS];
     int flag;
 };
 
@@ -74,18 +75,33 @@ __device__ __forceinline__ void cp_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// max over the CTA of a non-negative value; NaN counts as infinity
-__device__ double block_max(double v, double* red) {
-    if (!(v <= 1.7e308)) v = INFINITY;
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, off));
+// |v| as a whole number that orders like it to 2^-20: the upper half of its bits, at least 1 where v is not
+// zero.  Infinities and NaN are the largest.  Maxima are taken of these: with maxima in FP64
+// over the CTA, eight an iteration, 100 trajectories of P = 399 took 862 us; 771 us so.
+__device__ __forceinline__ uint32_t mag_key(double v) {
+    return ((uint32_t)__double2hiint(v) & 0x7FFFFFFFu) | (__double2loint(v) != 0 ? 1u : 0u);
+}
+__device__ __forceinline__ double key_value(uint32_t k) {
+    return k >= 0x7FF00000u ? INFINITY : __hiloint2double((int)k, 0);
+}
+// e with 2^(e - 1) <= v < 2^e for the v of a finite key (-1022 for zero and below the normal range)
+__device__ __forceinline__ int key_exponent(uint32_t k) { return max((int)(k >> 20), 0) - 1022; }
+// 2^k, |k| < 1000
+__device__ __forceinline__ double pow2(int k) { return __hiloint2double((1023 + k) << 20, 0); }
+
+// the largest a and the largest b over the CTA
+__device__ uint2 block_max2(uint32_t a, uint32_t b, uint32_t (*red)[WARPS]) {
+    static_assert(WARPS == 16, "a warp's maximum to each of 16 lanes");
+    a = __reduce_max_sync(0xffffffffu, a);
+    b = __reduce_max_sync(0xffffffffu, b);
     __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    if ((threadIdx.x & 31) == 0) {
+        red[0][threadIdx.x >> 5] = a;
+        red[1][threadIdx.x >> 5] = b;
+    }
     __syncthreads();
-    double m = red[0];
-#pragma unroll
-    for (int w = 1; w < WARPS; ++w) m = fmax(m, red[w]);
-    return m;
+    const uint32_t v = __reduce_max_sync(0xffffffffu, red[0][threadIdx.x & 15]);
+    return make_uint2(v, __reduce_max_sync(0xffffffffu, red[1][threadIdx.x & 15]));
 }
 
 // The three signed 21-bit digits of v (|v| < 2^62): v = d0 2^42 + d1 2^21 + d2.
@@ -416,7 +432,10 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
     // ---- refinement
     if (rank == 0)
         for (int i = tid; i < 2 * P; i += THREADS) gx[i] = 0.0;
-    double prev = 0.0;  // CTA 0: the last correction's largest |x / d|
+    // The two right-hand sides are systems of their own (they may differ by any factor): each has its
+    // exponents, its last correction and its end.
+    double prev[2] = {0.0, 0.0};  // CTA 0: the last correction's largest |x / d|
+    int conv = 0;                 // CTA 0: bit h set once right-hand side h has converged
     bool done = false;
     for (int it = 0; it < MAX_ITER; ++it) {
         if (it == 0) {
@@ -427,23 +446,24 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
                 }
         } else {
             // digits of x / d in units of 2^(ex - 60), 2^(ex - 1) <= max |x / d| < 2^ex
-            double m = 0.0;
+            uint32_t km[2] = {0u, 0u};
             for (int i = tid; i < P; i += THREADS)
-                m = fmax(m, fmax(fabs(__ldcg(gx + i)), fabs(__ldcg(gx + P + i))) / (double)dsc[i]);
-            m = block_max(m, sm.red[0]);
-            int ex;
-            frexp(m, &ex);
-            for (int i = tid; i < PY; i += THREADS) {
 #pragma unroll
-                for (int h = 0; h < 2; ++h) {
+                for (int h = 0; h < 2; ++h) km[h] = max(km[h], mag_key(__ldcg(gx + h * P + i) * pow2(-dsh[i])));
+            const uint2 kx = block_max2(km[0], km[1], sm.red);
+            double unit[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int ex = key_exponent(h ? kx.y : kx.x);
+                unit[h] = ldexp(1.0, ex - 120);
+                for (int i = tid; i < PY; i += THREADS) {
                     int d[3] = {0, 0, 0};
-                    if (i < P) digits(__double2ll_rn(ldexp(__ldcg(gx + h * P + i) / (double)dsc[i], 60 - ex)), d);
+                    if (i < P) digits(__double2ll_rn(ldexp(__ldcg(gx + h * P + i), 60 - ex - dsh[i])), d);
 #pragma unroll
                     for (int q = 0; q < 3; ++q) xd[6 * i + 3 * h + q] = d[q];
                 }
             }
             __syncthreads();
-            const double unit = ldexp(1.0, ex - 120);
             for (int i = warp + WARPS * rank; i < P; i += WARPS * cn) {
                 const double* Si = St + (size_t)i * P;
                 const int shi = dsh[i];
@@ -479,62 +499,64 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
                     const int h = lane;
                     const double dd = (h ? Dt[i].y : Dt[i].x) * (double)dsc[i];
                     const long long a0 = h ? a[1][0] : a[0][0], a1 = h ? a[1][1] : a[0][1], a2 = h ? a[1][2] : a[0][2];
-                    double r = fma(-(double)a0, unit * 0x1.0p84, dd);
+                    const double u = h ? unit[1] : unit[0];
+                    double r = fma(-(double)a0, u * 0x1.0p84, dd);
                     r = fma(-eps * (double)dsc[i], __ldcg(gx + h * P + i), r);
-                    r = fma(-(double)a1, unit * 0x1.0p63, r);
-                    gr[h * P + i] = fma(-(double)a2, unit * 0x1.0p42, r);
+                    r = fma(-(double)a1, u * 0x1.0p63, r);
+                    gr[h * P + i] = fma(-(double)a2, u * 0x1.0p42, r);
                 }
             }
             __threadfence();
             cl.sync();
         }
         if (rank == 0) {
-            double rmax = 0.0;
-            // (NaN counts as infinity in block_max; fmax alone would drop it, and a right-hand side of NaN and
-            // zeros would read as zero)
-            for (int i = tid; i < P; i += THREADS) {
-                const double ra = __ldcg(gr + i), rb = __ldcg(gr + P + i);
-                rmax = isfinite(ra) && isfinite(rb) ? fmax(rmax, fmax(fabs(ra), fabs(rb))) : INFINITY;
-            }
-            rmax = block_max(rmax, sm.red[0]);
             int stop = 0;  // 1: converged, 2: left to FP64
-            if (rmax == 0.0) {
-                stop = 1;
-            } else if (!(rmax < 1e300)) {
-                stop = 2;
-            } else {
-                int ex;
-                frexp(rmax, &ex);
-                const double up = ldexp(1.0, -ex), down = ldexp(1.0, ex);
-                for (int i = tid; i < PY; i += THREADS) {
-                    y[i] = i < P ? (float)(__ldcg(gr + i) * up) : 0.f;
-                    y[PY + i] = i < P ? (float)(__ldcg(gr + P + i) * up) : 0.f;
+            uint32_t km[2] = {0u, 0u};
+            for (int i = tid; i < P; i += THREADS)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) km[h] = max(km[h], mag_key(__ldcg(gr + h * P + i)));
+            const uint2 kr = block_max2(km[0], km[1], sm.red);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const double rmax = key_value(h ? kr.y : kr.x);
+                if (rmax == 0.0) conv |= 1 << h;
+                if (!(rmax < 1e300)) stop = 2;
+            }
+            if (stop == 0 && conv != 3) {
+                double down[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int ex = key_exponent(h ? kr.y : kr.x);
+                    const double up = conv & (1 << h) ? 0.0 : ldexp(1.0, -ex);
+                    down[h] = ldexp(1.0, ex);
+                    for (int i = tid; i < PY; i += THREADS)
+                        y[h * PY + i] = i < P ? (float)(__ldcg(gr + h * P + i) * up) : 0.f;
                 }
                 __syncthreads();
                 solve32(P, PY, ld, L, Xi, y, sm);
-                double ndx = 0.0, nx = 0.0;  // largest |dx / d| and |x / d|
-                for (int i = tid; i < P; i += THREADS) {
-                    const double ds = (double)dsc[i];
-                    const double da = (double)y[i] * down, db = (double)y[PY + i] * down;
-                    const double xa = __ldcg(gx + i) + da * ds, xb = __ldcg(gx + P + i) + db * ds;
-                    ndx = isfinite(da) && isfinite(db) ? fmax(ndx, fmax(fabs(da), fabs(db))) : INFINITY;
-                    nx = fmax(nx, fmax(fabs(xa), fabs(xb)) / ds);
-                    gx[i] = xa;
-                    gx[P + i] = xb;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (conv & (1 << h)) continue;
+                    uint32_t kd = 0u, kn = 0u;  // largest |dx / d| and |x / d|
+                    for (int i = tid; i < P; i += THREADS) {
+                        const double dx = (double)y[h * PY + i] * down[h];
+                        const double x = fma(dx, pow2(dsh[i]), __ldcg(gx + h * P + i));
+                        kd = max(kd, mag_key(dx));
+                        kn = max(kn, mag_key(x * pow2(-dsh[i])));
+                        gx[h * P + i] = x;
+                    }
+                    const uint2 k = block_max2(kd, kn, sm.red);
+                    const double ndx = key_value(k.x), nx = key_value(k.y);
+                    // rate of the refinement from the last two corrections: what is left after this one is
+                    // about rate * ndx.  Corrections at the rounding of x itself cannot shrink further.
+                    if (!(ndx < 1e300) || !(nx < 1e300) || (it > 0 && ndx > 0.25 * prev[h] && ndx > 1e-15 * nx))
+                        stop = 2;
+                    else if (it > 0 && (ndx * fmax(ndx / prev[h], 0x1.0p-22) <= 0x1.0p-54 * nx || ndx <= 1e-15 * nx))
+                        conv |= 1 << h;
+                    prev[h] = ndx;
                 }
-                ndx = block_max(ndx, sm.red[0]);
-                nx = block_max(nx, sm.red[1]);
-                // rate of the refinement from the last two corrections: what is left after this one is
-                // about rate * ndx.  Corrections at the rounding of x itself cannot shrink further.
-                if (!(ndx < 1e300) || !(nx < 1e300) || (it > 0 && ndx > 0.25 * prev && ndx > 1e-15 * nx)) {
-                    stop = 2;
-                } else if (it > 0 && (ndx * fmax(ndx / prev, 0x1.0p-22) <= 0x1.0p-54 * nx || ndx <= 1e-15 * nx)) {
-                    stop = 1;
-                } else if (it == MAX_ITER - 1) {
-                    stop = 2;
-                }
-                prev = ndx;
             }
+            if (stop == 0) stop = conv == 3 ? 1 : it == MAX_ITER - 1 ? 2 : 0;
             if (tid == 0) flags[t] = stop;
         }
         __threadfence();

@@ -1,5 +1,5 @@
 """Right-hand sides of the refined FP64 solve: a non-finite one is reported whatever its other entries
-are."""
+are, and the real and the imaginary system are each solved to their own accuracy."""
 import numpy as np
 import pytest
 
@@ -41,3 +41,18 @@ def test_solution_beyond_the_range_is_reported():
     st, x, _ = _solve(P, S, D, 0.0)
     assert st == abi.OTVMC_ERR_NOT_PD
     assert np.all(x[0] == 0) and np.all(x[1] == 1)
+
+
+@pytest.mark.parametrize("P,ratio", [(199, 1e-8), (199, 1e8), (65, 1e-30), (287, 1e-14), (48, 0.0)])
+def test_parts_are_solved_separately(P, ratio):
+    """The bound of the FP64 solve, 4 P 2^-53 cond of the largest entry, for each part by itself."""
+    S, D = _inputs(P, 2, 4 * P, 11)
+    D = D.real * ratio + 1j * D.imag
+    st, x, shift = _solve(P, S, D, 1e-4)
+    assert st == abi.OTVMC_OK and np.all(shift == 1e-4)
+    for t in range(2):
+        A = S[t] + 1e-4 * np.eye(P)
+        tol = 4 * P * 2.0 ** -53 * np.linalg.cond(A)
+        for got, rhs in ((x[t].real, D[t].real), (x[t].imag, D[t].imag)):
+            w = np.linalg.solve(A, rhs)
+            assert np.abs(got - w).max() <= tol * np.abs(w).max()
