@@ -9,26 +9,30 @@
 //      cluster take chunks of 256 rows of the update C = A - L L_b^T (SIMT, 4 x 4 per thread,
 //      operands staged by asynchronous copies); one warp of CTA 0 factors and inverts the
 //      diagonal tile (factor32); the CTAs multiply their rows of C by the inverse.
-//   3. r = D - A x (rows over the warps of the cluster), dx from the FP32 factor (CTA 0), x += dx in
-//      FP64, until the next correction, foretold from the last two, is below 2^-54 of x, for the real
-//      and the imaginary system separately (a part 1e-8 of the other was left at 3e-11 of itself).  The
-//      residual is taken from whole numbers: d S d and x / d as 63-bit fixed point in three signed
-//      digits of 21 bits, the six leading digit products summed exactly in 64-bit integers.  Its
-//      error is about 2^-61 |x|, below what an FP64 dot product leaves (2^-53 |S| |x|), so that the
-//      solution is rounded from a value correct to a few 2^-53 wherever the refinement converges.
+//   3. dx from the FP32 factor (CTA 0), x += dx in FP64, r -= A dx (rows over the warps of the cluster), from
+//      x = 0 and r = D until the next correction, foretold from the last two, is below 2^-54 of x; the real
+//      and the imaginary system separately (they may differ by any factor).  A dx is taken from whole
+//      numbers: d S d in units of 2^-60 as three digits of 21 bits, dx / d rounded to 28 bits of its largest
+//      entry (the rounded dx is the correction), their products summed exactly in 64-bit integers, so
+//      that r is that of the sum of the corrections to about 2^-73 of D.  The solution is that sum rounded to
+//      FP64.  All that is lost are the bits of d S d beyond 2^-60 in entries below 2^-8 (P = 399,
+//      conditions 3e3 to 5e3: 2e-16 of the largest entry; with x in three digits and the six largest of
+//      their nine products 1e-14; an FP64 Cholesky 2e-14 to 6e-14).
 //
 // Bound: the FP64 rate of these GPUs is 1/64 of the FP32 one.  The O(P^3) part runs in FP32; of the
-// residuals' O(P^2), the integer form takes about 45 integer instructions an entry, half the time
-// of two FP64 multiply-adds.
+// residuals' O(P^2), the integer form takes about 30 integer instructions an entry, less than half the
+// time of two FP64 multiply-adds.
 //
-// 100 trajectories of P = 399: 0.80 ms (8.8 ms with the FP64 factorization, one CTA per
-// trajectory); 8 of P = 528: 0.86 ms (15 ms).  Below P = 48 the factor and its inverses do not fit
+// 100 trajectories of P = 399: 0.75 ms (0.80 ms with the residual from all of x; 8.8 ms with the FP64
+// factorization, one CTA per trajectory); 8 of P = 528: 0.80 ms (15 ms).  Below P = 48 the factor and its inverses do not fit
 // the scratch that the FP64 factorization needs anyway.
 //
 // A trajectory is left to the FP64 factorization (flag 1) when a pivot of the FP32 one is not
-// clear of the shift test's threshold by the FP32 rounding (so that the decision to raise the
-// shift is always taken in FP64), when an entry is not finite, or when the refinement does not
-// converge.
+// clear of the shift test's threshold by several times the FP32 rounding to be expected in it (so
+// that the decision to raise the shift is FP64's; an estimate, not a bound: the worst case of a pivot's
+// rounding grows as P, not sqrt(P)), when an entry is not finite, or when the refinement does not
+// converge.  Such a call pays for the attempt as well: 9.1 ms for 8.8 ms at 100 trajectories of P = 399 on 300
+// samples and a shift of 1e-6, whose pivots end near the shift (1.4 ms at a shift of 1e-4, which converges).
 #include <cooperative_groups.h>
 
 #include "chol_tile.cuh"
@@ -61,6 +65,7 @@ struct alignas(16) Smem {  // its size a multiple of 16: float4 vectors follow i
     float scr[4 * TB];
     float t[2][TB];
     uint32_t red[2][WARPS];
+    int zex[2];  // CTA 0: exponents of the units of the corrections
     int flag;
 };
 
@@ -102,16 +107,6 @@ __device__ uint2 block_max2(uint32_t a, uint32_t b, uint32_t (*red)[WARPS]) {
     __syncthreads();
     const uint32_t v = __reduce_max_sync(0xffffffffu, red[0][threadIdx.x & 15]);
     return make_uint2(v, __reduce_max_sync(0xffffffffu, red[1][threadIdx.x & 15]));
-}
-
-// The three signed 21-bit digits of v (|v| < 2^62): v = d0 2^42 + d1 2^21 + d2.
-__device__ __forceinline__ void digits(long long v, int (&d)[3]) {
-    const int d2 = (int)((unsigned)v << 11) >> 11;
-    v = (v - d2) >> 21;
-    const int d1 = (int)((unsigned)v << 11) >> 11;
-    d[2] = d2;
-    d[1] = d1;
-    d[0] = (int)((v - d1) >> 21);
 }
 
 // The three 21-bit digits of s 2^(60 + sh), truncated towards zero, each with the sign of s: exact
@@ -269,14 +264,14 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
     const size_t ld = ld_of(P), PP = (size_t)P * P;
     float* dsc = reinterpret_cast<float*>(smraw + sizeof(Smem));  // [PY] scales
     float* y = dsc + PY;                                         // [2][PY] right-hand sides of the FP32 solve
-    int* xd = reinterpret_cast<int*>(y + 2 * PY);                // [PY][2][3] digits of x / d
-    int* dsh = xd + 6 * PY;                                      // [PY] log2 of the scales
+    int2* zq = reinterpret_cast<int2*>(y + 2 * PY);              // [PY] the last correction over d, whole numbers
+    int* dsh = reinterpret_cast<int*>(zq + PY);                  // [PY] log2 of the scales
     const double* St = S + (size_t)t * PP;
     const double2* Dt = D + (size_t)t * P;
     // an odd P leaves the trajectory's scratch at 8 bytes past a multiple of 16
     float* L = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(Lws + (size_t)t * PP) + 15) & ~(uintptr_t)15);
     float* Xi = L + (size_t)P * ld;          // [nblk][TB][TB]
-    double* gx = xws + (size_t)t * 4 * P;    // [2][P] x, then [2][P] r, shared by the cluster
+    double* gx = xws + (size_t)t * 4 * P;    // [2][P] x (CTA 0), then [2][P] r, shared by the cluster
     double* gr = gx + 2 * P;
 
     // scales; a diagonal entry that is not a positive normal number goes to FP64
@@ -312,7 +307,7 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
                 for (int v = 0; v < 4; ++v) acc[u][v] = 0.f;
             const int nk = jb / KC;  // KC divides TB
             auto stage = [&](int s, int k0) {
-                // 16 columns x 256 rows (64 pieces of 16 bytes each), 16 x 32 rows of the block
+                // KC columns x 256 rows (64 pieces of 16 bytes each), KC x 32 rows of the block
 #pragma unroll
                 for (int e = tid; e < KC * (RC / 4); e += THREADS) {
                     const int kk = e / (RC / 4), i4 = 4 * (e % (RC / 4));
@@ -445,23 +440,12 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
                     gr[P + i] = Dt[i].y * (double)dsc[i];
                 }
         } else {
-            // digits of x / d in units of 2^(ex - 60), 2^(ex - 1) <= max |x / d| < 2^ex
-            uint32_t km[2] = {0u, 0u};
-            for (int i = tid; i < P; i += THREADS)
-#pragma unroll
-                for (int h = 0; h < 2; ++h) km[h] = max(km[h], mag_key(__ldcg(gx + h * P + i) * pow2(-dsh[i])));
-            const uint2 kx = block_max2(km[0], km[1], sm.red);
-            double unit[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int ex = key_exponent(h ? kx.y : kx.x);
-                unit[h] = ldexp(1.0, ex - 120);
-                for (int i = tid; i < PY; i += THREADS) {
-                    int d[3] = {0, 0, 0};
-                    if (i < P) digits(__double2ll_rn(ldexp(__ldcg(gx + h * P + i), 60 - ex - dsh[i])), d);
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) xd[6 * i + 3 * h + q] = d[q];
-                }
+            // r -= A dx, the correction from CTA 0
+            const Smem* sm0 = cl.map_shared_rank(&sm, 0);
+            const int ze[2] = {sm0->zex[0], sm0->zex[1]};
+            if (rank != 0) {
+                const int2* zq0 = cl.map_shared_rank(zq, 0);
+                for (int i = tid; i < P; i += THREADS) zq[i] = zq0[i];
             }
             __syncthreads();
             for (int i = warp + WARPS * rank; i < P; i += WARPS * cn) {
@@ -474,17 +458,11 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
                 for (int j = lane; j < P; j += 32) {
                     int sd[3];
                     digits_of(Si[j], shi + dsh[j], sd);
-                    const int2* xj = reinterpret_cast<const int2*>(xd + 6 * j);
-                    const int2 x0 = xj[0], x1 = xj[1], x2 = xj[2];
-                    const int xv[2][3] = {{x0.x, x0.y, x1.x}, {x1.y, x2.x, x2.y}};
+                    const int2 z = zq[j];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        a[h][0] += (long long)sd[0] * xv[h][0];
-                        a[h][1] += (long long)sd[0] * xv[h][1];
-                        a[h][1] += (long long)sd[1] * xv[h][0];
-                        a[h][2] += (long long)sd[0] * xv[h][2];
-                        a[h][2] += (long long)sd[1] * xv[h][1];
-                        a[h][2] += (long long)sd[2] * xv[h][0];
+                    for (int q = 0; q < 3; ++q) {
+                        a[0][q] += (long long)sd[q] * z.x;
+                        a[1][q] += (long long)sd[q] * z.y;
                     }
                 }
 #pragma unroll
@@ -494,16 +472,16 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
 #pragma unroll
                         for (int q = 0; q < 3; ++q) a[h][q] += __shfl_xor_sync(0xffffffffu, a[h][q], off);
                 if (lane < 2) {
-                    // d_i r_i = d_i D_i - sum - eps d_i x_i, the largest terms first: the first
-                    // difference is small already, and the digit sums (below 2^53) convert exactly
-                    const int h = lane;
-                    const double dd = (h ? Dt[i].y : Dt[i].x) * (double)dsc[i];
+                    // the sum, a whole number below 2^103, in two parts that convert exactly, largest first: the
+                    // difference is small already
+                    const int h = lane, zi = h ? zq[i].y : zq[i].x, zx = h ? ze[1] : ze[0];
                     const long long a0 = h ? a[1][0] : a[0][0], a1 = h ? a[1][1] : a[0][1], a2 = h ? a[1][2] : a[0][2];
-                    const double u = h ? unit[1] : unit[0];
-                    double r = fma(-(double)a0, u * 0x1.0p84, dd);
-                    r = fma(-eps * (double)dsc[i], __ldcg(gx + h * P + i), r);
-                    r = fma(-(double)a1, u * 0x1.0p63, r);
-                    gr[h * P + i] = fma(-(double)a2, u * 0x1.0p42, r);
+                    const __int128 N = ((__int128)a0 << 42) + ((__int128)a1 << 21) + a2;
+                    const long long hi = (long long)(N >> 53), lo = (long long)(N - ((__int128)hi << 53));
+                    const double u = ldexp(1.0, zx), d = pow2(shi);
+                    double r = fma(-(double)hi, u * 0x1.0p-7, __ldcg(gr + h * P + i));
+                    r = fma(-(double)lo, u * 0x1.0p-60, r);
+                    gr[h * P + i] = fma(-eps * d * d * u, (double)zi, r);
                 }
             }
             __threadfence();
@@ -520,40 +498,58 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
             for (int h = 0; h < 2; ++h) {
                 const double rmax = key_value(h ? kr.y : kr.x);
                 if (rmax == 0.0) conv |= 1 << h;
-                if (!(rmax < 1e300)) stop = 2;
+                // (the units of r, a 2^-167 of it at the end, stay normal numbers)
+                else if (!(rmax < 0x1p800) || (it == 0 && rmax < 0x1p-800)) stop = 2;
             }
             if (stop == 0 && conv != 3) {
-                double down[2];
+                int rex[2];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    const int ex = key_exponent(h ? kr.y : kr.x);
-                    const double up = conv & (1 << h) ? 0.0 : ldexp(1.0, -ex);
-                    down[h] = ldexp(1.0, ex);
+                    rex[h] = key_exponent(h ? kr.y : kr.x);
+                    const double up = conv & (1 << h) ? 0.0 : ldexp(1.0, -rex[h]);
                     for (int i = tid; i < PY; i += THREADS)
                         y[h * PY + i] = i < P ? (float)(__ldcg(gr + h * P + i) * up) : 0.f;
                 }
                 __syncthreads();
                 solve32(P, PY, ld, L, Xi, y, sm);
+                // the correction over d in units of 2^(ex - 27), 2^(ex - 1) <= its largest entry < 2^ex
+                uint32_t kz[2] = {0u, 0u};  // (bits of a float's magnitude order like it)
+                for (int i = tid; i < P; i += THREADS)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) kz[h] = max(kz[h], __float_as_uint(y[h * PY + i]) & 0x7FFFFFFFu);
+                const uint2 kd = block_max2(kz[0], kz[1], sm.red);
+                uint32_t kn[2] = {0u, 0u};
+                double ndx[2];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t k = h ? kd.y : kd.x;
+                    const int ex = (int)(k >> 23) - 126;
+                    const bool live = !(conv & (1 << h));
+                    if (live && (ex < -60 || ex > 60)) stop = 2;  // (a correction of zeros, or not finite, among them)
+                    const float up = live && stop == 0 ? __uint_as_float((uint32_t)(127 + 27 - ex) << 23) : 0.f;
+                    const double unit = live ? ldexp(1.0, rex[h] + ex - 27) : 0.0;
+                    ndx[h] = ldexp((double)__uint_as_float(k), rex[h]);
+                    if (tid == 0) sm.zex[h] = rex[h] + ex - 27;
+                    for (int i = tid; i < P; i += THREADS) {
+                        const int z = __float2int_rn(y[h * PY + i] * up);
+                        (h ? zq[i].y : zq[i].x) = z;
+                        const double x = fma((double)z, unit * pow2(dsh[i]), __ldcg(gx + h * P + i));
+                        kn[h] = max(kn[h], mag_key(x * pow2(-dsh[i])));
+                        gx[h * P + i] = x;
+                    }
+                }
+                const uint2 kx = block_max2(kn[0], kn[1], sm.red);
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     if (conv & (1 << h)) continue;
-                    uint32_t kd = 0u, kn = 0u;  // largest |dx / d| and |x / d|
-                    for (int i = tid; i < P; i += THREADS) {
-                        const double dx = (double)y[h * PY + i] * down[h];
-                        const double x = fma(dx, pow2(dsh[i]), __ldcg(gx + h * P + i));
-                        kd = max(kd, mag_key(dx));
-                        kn = max(kn, mag_key(x * pow2(-dsh[i])));
-                        gx[h * P + i] = x;
-                    }
-                    const uint2 k = block_max2(kd, kn, sm.red);
-                    const double ndx = key_value(k.x), nx = key_value(k.y);
+                    const double nx = key_value(h ? kx.y : kx.x);  // largest |x / d|
                     // rate of the refinement from the last two corrections: what is left after this one is
                     // about rate * ndx.  Corrections at the rounding of x itself cannot shrink further.
-                    if (!(ndx < 1e300) || !(nx < 1e300) || (it > 0 && ndx > 0.25 * prev[h] && ndx > 1e-15 * nx))
+                    if (!(ndx[h] < 1e300) || !(nx < 1e300) || (it > 0 && ndx[h] > 0.25 * prev[h] && ndx[h] > 1e-15 * nx))
                         stop = 2;
-                    else if (it > 0 && (ndx * fmax(ndx / prev[h], 0x1.0p-22) <= 0x1.0p-54 * nx || ndx <= 1e-15 * nx))
+                    else if (it > 0 && (ndx[h] * fmax(ndx[h] / prev[h], 0x1.0p-22) <= 0x1.0p-54 * nx || ndx[h] <= 1e-15 * nx))
                         conv |= 1 << h;
-                    prev[h] = ndx;
+                    prev[h] = ndx[h];
                 }
             }
             if (stop == 0) stop = conv == 3 ? 1 : it == MAX_ITER - 1 ? 2 : 0;
@@ -579,14 +575,15 @@ __global__ void __launch_bounds__(THREADS, 1) solve_ref_kernel(int P, double eps
 static_assert(sizeof(Smem) % 16 == 0, "the vectors behind Smem are read as float4");
 static size_t smem_bytes(int P) {
     const size_t PY = (size_t)((P + TB - 1) / TB) * TB;
-    return sizeof(Smem) + PY * 4 + 2 * PY * 4 + 6 * PY * 4 + PY * 4;
+    return sizeof(Smem) + PY * 4 + 2 * PY * 4 + PY * 8 + PY * 4;
 }
 
 }  // namespace solref
 
-// P up to what the vectors of one trajectory leave of a CTA's shared memory (40 bytes a parameter),
-// and from where the FP32 factor and the tiles' inverses fit the P^2 doubles of scratch.
-bool solve_ref_ok(int P) { return P >= 48 && solref::smem_bytes(P) <= 220 * 1024; }
+// From where the FP32 factor and the tiles' inverses fit the P^2 doubles of scratch, to where the vectors of
+// 40 bytes a parameter of its first form fitted a CTA's shared memory (those of now, 24 bytes, would up to about
+// P = 5900: not measured).
+bool solve_ref_ok(int P) { return P >= 48 && P <= 3520; }
 
 // flags[t] = 0: solved; 1: left to the FP64 factorization.  Lws: P^2 doubles per trajectory, xws:
 // 4 P doubles per trajectory.

@@ -1,5 +1,6 @@
 """Right-hand sides of the refined FP64 solve: a non-finite one is reported whatever its other entries
-are, and the real and the imaginary system are each solved to their own accuracy."""
+are, the real and the imaginary system are each solved to their own accuracy, and a solution is
+correct to the rounding of FP64."""
 import numpy as np
 import pytest
 
@@ -55,4 +56,25 @@ def test_parts_are_solved_separately(P, ratio):
         tol = 4 * P * 2.0 ** -53 * np.linalg.cond(A)
         for got, rhs in ((x[t].real, D[t].real), (x[t].imag, D[t].imag)):
             w = np.linalg.solve(A, rhs)
+            assert np.abs(got - w).max() <= tol * np.abs(w).max()
+
+
+@pytest.mark.parametrize("P,ns,eps", [(99, 110, 1e-4), (199, 230, 1e-4), (399, 440, 1e-3), (399, 420, 1e-4)])
+def test_solution_is_correct_to_its_rounding(P, ns, eps):
+    """Against the solution in extended precision, at conditions of 1e3 to 5e3 where a plain FP64 solve
+    is off by 5e-15 to 6e-14.  Bound: the rounding of x and what is left after the last correction, 2^-53
+    each, and the residual's error, entries of the scaled S below 2^-8 cut at 2^-60, through the inverse."""
+    S, D = _inputs(P, 2, ns, 21)
+    st, x, shift = _solve(P, S, D, eps)
+    assert st == abi.OTVMC_OK and np.all(shift == eps)
+    L = np.longdouble
+    for t in range(2):
+        A = S[t].astype(L) + L(eps) * np.eye(P).astype(L)
+        inv = np.linalg.inv(A.astype(np.float64))
+        d = 2.0 ** -((np.floor(np.log2(np.diag(S[t]) + eps)).astype(int) + 1) >> 1)
+        tol = 2.0 ** -52 + 2.0 ** -60 * np.linalg.norm(inv / np.outer(d, d), 2)
+        for got, rhs in ((x[t].real, D[t].real), (x[t].imag, D[t].imag)):
+            w = np.zeros(P, L)
+            for _ in range(10):
+                w = w + inv @ (rhs.astype(L) - A @ w).astype(np.float64)
             assert np.abs(got - w).max() <= tol * np.abs(w).max()
