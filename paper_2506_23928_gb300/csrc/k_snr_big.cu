@@ -289,11 +289,11 @@ __device__ __forceinline__ double to_double(__int128 v) {
 __global__ void __launch_bounds__(256, 2) snr_wgram_kernel(OShape o, int ns, const uint64_t* __restrict__ spins,
                                                         const double2* __restrict__ v,
                                                         const double* __restrict__ obar, double* __restrict__ M) {
-    const int t = blockIdx.y, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    int J = (int)((sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f) * 0.5f);
-    while ((J + 1) * (J + 2) / 2 <= (int)blockIdx.x) ++J;
-    while (J * (J + 1) / 2 > (int)blockIdx.x) --J;
-    const int I = blockIdx.x - J * (J + 1) / 2, r0 = I * WG, c0 = J * WG, P = o.P, W = o.W;
+    const int t = blockIdx.x, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    int J = (int)((sqrtf(8.f * (float)blockIdx.y + 1.f) - 1.f) * 0.5f);
+    while ((J + 1) * (J + 2) / 2 <= (int)blockIdx.y) ++J;
+    while (J * (J + 1) / 2 > (int)blockIdx.y) --J;
+    const int I = blockIdx.y - J * (J + 1) / 2, r0 = I * WG, c0 = J * WG, P = o.P, W = o.W;
     __shared__ __align__(16) int As[WK][WG];           // O of the tile's rows
     __shared__ __align__(16) int B1[WK][WG], B0[WK][WG];  // O of its columns times the digits of w
     __shared__ uint64_t sw[WK][4];
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(QL_THREADS, 1) snr_ql_kernel(int P, double* __
 __global__ void __launch_bounds__(256) snr_var_kernel(int P, const double* __restrict__ Xws, double* Mws) {
     constexpr int BR = 32, BJ = 64, BI = 16;
     __shared__ double As[BI][BR + 1], Bs[BI][BJ];
-    const int t = blockIdx.y, k0 = blockIdx.x * BR, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const int t = blockIdx.x, k0 = blockIdx.y * BR, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     const double* X = Xws + (size_t)t * P * P;
     double* M = Mws + (size_t)t * P * P;
     double q2[2] = {0.0, 0.0};
@@ -745,11 +745,12 @@ cudaError_t launch_snr_big(const otvmc_ansatz* a, int ntraj, int ns, const uint6
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(snr_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * P * (int)sizeof(double));
     if (e != cudaSuccess) return e;
+    // (the trajectories along x: a grid's other dimensions end at 65535)
     const int nt = (P + WG - 1) / WG;
     snr_tri_kernel<<<ntraj, SNRB_THREADS, smem_tri, s>>>(P, S, Aws, Xws);
-    snr_wgram_kernel<<<dim3(nt * (nt + 1) / 2, ntraj), 256, 0, s>>>(o, ns, spins, v, obar, Aws);
+    snr_wgram_kernel<<<dim3(ntraj, nt * (nt + 1) / 2), 256, 0, s>>>(o, ns, spins, v, obar, Aws);
     snr_ql_kernel<<<ntraj, QL_THREADS, smem_ql, s>>>(P, Aws, Xws, status);
-    snr_var_kernel<<<dim3((P + 31) / 32, ntraj), 256, 0, s>>>(P, Xws, Aws);
+    snr_var_kernel<<<dim3(ntraj, (P + 31) / 32), 256, 0, s>>>(P, Xws, Aws);
     snr_final_kernel<<<ntraj, 256, 2 * P * (int)sizeof(double), s>>>(P, ns, D, thr, eps_svd, Aws, Xws, delta, lam);
     count_launch(5);
     return cudaGetLastError();
