@@ -301,10 +301,10 @@ OTVMC_API otvmc_status otvmc_solve_step(const otvmc_ansatz* ansatz, int ntraj, i
  * Jastrow and tied Jastrow ansaetze, FP64 throughout.  P <= 96: a cyclic Jacobi
  * eigen-decomposition in shared memory, one CTA per trajectory.  Larger P (up to about 3000):
  * Householder tridiagonalisation of a copy of S in the workspace, the eigenvectors formed
- * explicitly and refined by the implicit QL iteration (shift from the leading 2 x 2 block), and
- * Var_x Q_k from M = sum_x |v_c|^2 O_c O_c^T (exact integer sums, |v_c|^2 to 46 bits of its largest
- * value) as v_k^T M v_k; this costs O(P^3) FP64 work per trajectory and O(ns P^2) integer work.  Inputs: S_d [ntraj][P][P] full FP64 S (otvmc_build_S_F), obar_d
- * [ntraj][P], spins_d [ntraj][ns][W], v_d [ntraj][ns] double2 (otvmc_local_estimators), D_d
+ * explicitly and refined by the implicit QL iteration (shift from the leading 2 x 2 block), then one
+ * pass over the samples, which sums Q_k and |Q_k|^2 (V^T O_c in exact integers, V to 2^-61); this
+ * costs O(P^3) FP64 work per trajectory and O(ns P^2) integer work.  Inputs: S_d [ntraj][P][P] full
+ * FP64 S (otvmc_build_S_F), obar_d [ntraj][P], spins_d [ntraj][ns][W], v_d [ntraj][ns] double2 (otvmc_local_estimators), D_d
  * [ntraj][P] double2.  work_bytes >= otvmc_snr_workspace_bytes(ansatz, ntraj) (256 bytes of
  * status for P <= 96, plus 2 P^2 doubles per trajectory beyond).  Outputs: delta_d [ntraj][P]
  * double2; lambda_d (optional) [ntraj][P] eigenvalues, unordered.  A decomposition that has

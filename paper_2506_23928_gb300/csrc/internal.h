@@ -272,7 +272,7 @@ int lj_operand_rows(const otvmc_ansatz* a);
 constexpr int SNR_PMAX = 96;
 constexpr double SNR_EPS_SVD = 1e-12;
 size_t snr_smem_bytes(int P);
-// the same filter for larger P: Householder tridiagonalisation, implicit QL, weighted Gram matrix (k_snr_big.cu)
+// the same filter for larger P: Householder tridiagonalisation, implicit QL, sample pass (k_snr_big.cu)
 size_t snr_big_ws_bytes(int ntraj, int P);
 bool snr_big_fits(int P);
 cudaError_t launch_snr_big(const otvmc_ansatz* a, int ntraj, int ns, const uint64_t* spins, const double* S,

@@ -9,25 +9,22 @@
 //          H_k = I - tau_k v_k v_k^T acting on indices k+1 .. P-1 (v_k kept in column k of A); then
 //          Q^T explicitly, as X = H_{P-3}, X <- X H_k for k = P-4 .. 0, each step touching only the
 //          trailing block that H_k acts on.  One CTA per trajectory.
-//   wgram  M = sum_x w(x) O_c(x) O_c(x)^T, w = |v_c|^2, into A's place: Var_x Q_k = v_k^T M v_k / ns -
-//          |rho_k|^2, which takes P^2 products per sample once for all k, half of them by symmetry,
-//          in place of the P^2 FP64 products of the projections y_k(x).  w as a 46-bit integer in two
-//          digits of 23 bits, O as the small integer that it is: every product and sum is exact in
-//          64-bit integers, which run at 16 times the FP64 rate.  One CTA per 64 x 64 tile.
 //   ql     the implicit QL iteration with the shift from the leading 2 x 2 block on T (d, e), every
 //          plane rotation applied to the rows of X, so that at the end row k of X is the eigenvector
 //          of eigenvalue d_k (X = V^T); eigenvalues to an absolute accuracy of a few eps ||S||, as a
 //          dense symmetric eigensolver gives them.  One CTA per trajectory: one warp runs the scalar
 //          recurrence of a sweep while eight apply the rotations of the sweep before.
-//   var    v_k^T M v_k, an FP64 product per 32 eigenvectors.
+//   mean   the means of O along the eigenvectors and of v.
+//   pass   Q_k of every sample from whole numbers, summed with |Q_k|^2: P^2 products per sample in two 32-bit
+//          digits of the eigenvectors, which run at 16 times the FP64 rate.
 //   final  rho, the filter and the back-projection.
 // Bound: FP64 at 2 multiply-adds per cycle and SM (tri: about 5/3 P^3 of them, ql: 2 per rotation and
-// column, about 3 P^3, var: P^3), and in ql the chain of the recurrence (about 0.85 P^2 rotations).
+// column, about 3 P^3), and in ql the chain of the recurrence (about 0.85 P^2 rotations).
 // 100 trajectories of P = 249, 4096 samples, in one kernel with FP64 projections of every sample
-// and the recurrence between the rotations: 321 ms; now 70 ms (tri
-// 12, wgram 8, ql 47, var 3; ql at 1,700 cycles a rotation of its recurrence, 730 of its columns).
-// A and X live in the caller's workspace (2 P^2 doubles per trajectory).  Only the upper triangle of M
-// is stored; d, e and v^T M v pass from launch to launch in the lower one (SnrScratch).
+// and the recurrence between the rotations: 321 ms; now 69.5 ms (tri
+// 12, ql 47, mean and pass 9.9; ql at 1,700 cycles a rotation of its recurrence, 730 of its columns).
+// A and X live in the caller's workspace (2 P^2 doubles per trajectory); the tridiagonal and then the eigenvalues
+// pass from launch to launch in A's last rows (SnrScratch), the sample pass's sums in its first (PassScratch).
 #include "common.cuh"
 
 namespace otvmc {
@@ -87,8 +84,8 @@ __device__ double block_sum(double v, double* red) {
     return s;
 }
 
-// d_k (then the eigenvalue) and e_k (then v_k^T M v_k) in the strict lower triangle of A, once the
-// reflectors there are no longer needed: rows P - 1 and P - 2, what does not fit in row P - 3.
+// d_k (then the eigenvalue) and e_k in the strict lower triangle of A, once the reflectors there are no
+// longer needed: rows P - 1 and P - 2, what does not fit in row P - 3.
 struct SnrScratch {
     double* A;
     int P;
@@ -234,202 +231,6 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_tri_kernel(int P, const d
         sc.d(i) = d[i];
         sc.e(i) = e[i];
     }
-}
-
-// ------------------------------------------------------------------------- weighted Gram
-constexpr int WG = 64;   // tile
-constexpr int WK = 32;   // samples per chunk
-constexpr int WBITS = 23;
-
-// O_k of a sample with spin words w[W] (shared memory): s_k, s_j s_l, or the sum over a tied group.
-struct OShape {
-    int n, W, P, nu;      // nu: parameters that are single spins or pairs
-    int d, pbc;           // tied distances d + 1 + (k - nu)
-    const int* pairs;     // pairs of the full Jastrow
-    const int* grp_pair;  // tied ansatz: the free groups' pairs (nullptr: parameter n + q is pair q)
-};
-__device__ __forceinline__ int o_value(const OShape& o, const uint64_t* w, int k) {
-    if (k < o.n) return spin_of(w, k);
-    if (k < o.nu) {
-        const int p = o.grp_pair ? __ldg(o.grp_pair + k - o.n) : k - o.n;
-        const int2 jl = __ldg(reinterpret_cast<const int2*>(o.pairs) + p);
-        return spin_of(w, jl.x) * spin_of(w, jl.y);
-    }
-    // all pairs at distance D: (pairs) - 2 (disagreeing ones), from the string shifted by D (rotated
-    // for a ring, where each pair half way round is met twice)
-    const int D = o.d + 1 + k - o.nu, m = o.pbc ? o.n : o.n - D;
-    int dis = 0;
-    for (int q = 0; q < o.W; ++q) {
-        const int left = m - 64 * q;
-        if (left <= 0) break;
-        uint64_t u = 0ull;
-        {
-            const int b = 64 * q + D, i = b >> 6, r = b & 63;
-            if (i < o.W) u = w[i] >> r;
-            if (r && i + 1 < o.W) u |= w[i + 1] << (64 - r);
-        }
-        if (o.pbc) {  // bits n - D and up take the string's first bits
-            const int b = 64 * q - (o.n - D), i = b >> 6, r = b & 63;  // (arithmetic shift: b may be negative)
-            if (i >= 0 && i < o.W) u |= w[i] >> r;
-            if (i + 1 >= 0 && i + 1 < o.W && r) u |= w[i + 1] << (64 - r);
-        }
-        const uint64_t mask = left >= 64 ? ~0ull : (1ull << left) - 1ull;
-        dis += __popcll((w[q] ^ u) & mask);
-    }
-    return o.pbc && 2 * D == o.n ? m / 2 - dis : m - 2 * dis;
-}
-
-__device__ __forceinline__ double to_double(__int128 v) {
-    const long long hi = (long long)(v >> 53), lo = (long long)(v - ((__int128)hi << 53));
-    // (hi may take more than 53 bits: then its conversion is the one rounding that counts)
-    return fma((double)hi, 9007199254740992.0, (double)lo);
-}
-
-// The upper triangle of M, a 64 x 64 tile per CTA.
-__global__ void __launch_bounds__(256, 2) snr_wgram_kernel(OShape o, int ns, const uint64_t* __restrict__ spins,
-                                                        const double2* __restrict__ v,
-                                                        const double* __restrict__ obar, double* __restrict__ M) {
-    const int t = blockIdx.x, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    int J = (int)((sqrtf(8.f * (float)blockIdx.y + 1.f) - 1.f) * 0.5f);
-    while ((J + 1) * (J + 2) / 2 <= (int)blockIdx.y) ++J;
-    while (J * (J + 1) / 2 > (int)blockIdx.y) --J;
-    const int I = blockIdx.y - J * (J + 1) / 2, r0 = I * WG, c0 = J * WG, P = o.P, W = o.W;
-    __shared__ __align__(16) int As[WK][WG];           // O of the tile's rows
-    __shared__ __align__(16) int B1[WK][WG], B0[WK][WG];  // O of its columns times the digits of w
-    __shared__ uint64_t sw[WK][4];
-    __shared__ int q1s[WK], q0s[WK];
-    __shared__ double red[8];
-    __shared__ long long redl[16];
-    __shared__ long long mrow[2 * WG][2];              // sums of w O, digit sums, rows then columns
-    const double2* vt = v + (size_t)t * ns;
-    const uint64_t* sp = spins + (size_t)t * ns * W;
-    // mean of v, largest w
-    double sx = 0.0, sy = 0.0;
-    for (int x = tid; x < ns; x += 256) {
-        sx += vt[x].x;
-        sy += vt[x].y;
-    }
-    const double vbx = block_sum<8>(sx, red) / ns, vby = block_sum<8>(sy, red) / ns;
-    double wm = 0.0;
-    for (int x = tid; x < ns; x += 256) {
-        const double a = vt[x].x - vbx, b = vt[x].y - vby;
-        wm = fmax(wm, a * a + b * b);
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) wm = fmax(wm, __shfl_xor_sync(0xffffffffu, wm, off));
-    __syncthreads();
-    if ((tid & 31) == 0) red[tid >> 5] = wm;
-    __syncthreads();
-    wm = red[0];
-#pragma unroll
-    for (int i = 1; i < 8; ++i) wm = fmax(wm, red[i]);
-    int ex = 0;
-    if (wm > 0.0 && wm < 1e300) frexp(wm, &ex);  // wm < 2^ex
-    const int sh = 2 * WBITS - ex;
-    const double up = ldexp(1.0, sh < 1000 ? sh : 1000);
-
-    long long a1[4][4], a0[4][4], ws1 = 0, ws0 = 0, m1 = 0, m0 = 0;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) a1[a][b] = a0[a][b] = 0;
-    for (int x0 = 0; x0 < ns; x0 += WK) {
-        __syncthreads();
-        for (int e = tid; e < WK * W; e += 256) {
-            const int x = e / W, q = e - x * W;
-            sw[x][q] = x0 + x < ns ? sp[(size_t)(x0 + x) * W + q] : 0ull;
-        }
-        if (tid < WK) {
-            long long q = 0;
-            if (x0 + tid < ns) {
-                const double a = vt[x0 + tid].x - vbx, b = vt[x0 + tid].y - vby;
-                q = __double2ll_rn((a * a + b * b) * up);
-            }
-            const long long top = (1ll << (2 * WBITS)) - 1;  // a w just below 2^ex may round up to it
-            q = q < 0 ? 0 : q > top ? top : q;
-            q1s[tid] = (int)(q >> WBITS);
-            q0s[tid] = (int)(q & ((1ll << WBITS) - 1));
-        }
-        __syncthreads();
-        for (int e = tid; e < 2 * WK * WG; e += 256) {
-            const int x = (e >> 6) & (WK - 1), r = e & (WG - 1);
-            const bool col = e >= WK * WG;  // uniform over a warp
-            const int k = (col ? c0 : r0) + r;
-            const int val = k < P ? o_value(o, sw[x], k) : 0;
-            if (col) {
-                B1[x][r] = val * q1s[x];
-                B0[x][r] = val * q0s[x];
-            } else {
-                As[x][r] = val;
-            }
-        }
-        __syncthreads();
-        if (tid < WG) {  // sums of w O of the rows, then of the columns; of w by one thread
-#pragma unroll 4
-            for (int x = 0; x < WK; ++x) {
-                m1 += (long long)As[x][tid] * q1s[x];
-                m0 += (long long)As[x][tid] * q0s[x];
-            }
-        } else if (tid < 2 * WG) {
-#pragma unroll 4
-            for (int x = 0; x < WK; ++x) {
-                m1 += B1[x][tid - WG];
-                m0 += B0[x][tid - WG];
-            }
-        } else if (tid == 2 * WG) {
-            for (int x = 0; x < WK; ++x) {
-                ws1 += q1s[x];
-                ws0 += q0s[x];
-            }
-        }
-#pragma unroll 4
-        for (int x = 0; x < WK; ++x) {
-            const int4 av = *reinterpret_cast<const int4*>(&As[x][4 * ty]);
-            const int4 b1 = *reinterpret_cast<const int4*>(&B1[x][4 * tx]), b0 = *reinterpret_cast<const int4*>(&B0[x][4 * tx]);
-            const int ar[4] = {av.x, av.y, av.z, av.w}, u1[4] = {b1.x, b1.y, b1.z, b1.w}, u0[4] = {b0.x, b0.y, b0.z, b0.w};
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) {
-                    a1[a][b] += (long long)ar[a] * u1[b];
-                    a0[a][b] += (long long)ar[a] * u0[b];
-                }
-        }
-    }
-    if (tid < 2 * WG) {
-        mrow[tid][0] = m1;
-        mrow[tid][1] = m0;
-    } else if (tid == 2 * WG) {
-        redl[0] = ws1;
-        redl[1] = ws0;
-    }
-    __syncthreads();
-    // centred: sum w (O_i - obar_i)(O_j - obar_j), exactly through c = ns obar where that is whole (the
-    // column means of the samples), else in FP64
-    const __int128 Wt = ((__int128)redl[0] << WBITS) + redl[1];
-    const double down = ldexp(1.0, sh < 1000 ? -sh : -1000);
-    const double* ob = obar + (size_t)t * P;
-    double* Mt = M + (size_t)t * P * P;
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const int i = r0 + 4 * ty + a, j = c0 + 4 * tx + b;
-            if (i >= P || j >= P || i > j) continue;
-            const __int128 Mij = ((__int128)a1[a][b] << WBITS) + a0[a][b];
-            const __int128 mi = ((__int128)mrow[4 * ty + a][0] << WBITS) + mrow[4 * ty + a][1];
-            const __int128 mj = ((__int128)mrow[WG + 4 * tx + b][0] << WBITS) + mrow[WG + 4 * tx + b][1];
-            const double oi = ob[i], oj = ob[j];
-            const long long ci = __double2ll_rn(oi * ns), cj = __double2ll_rn(oj * ns);
-            double val;
-            if (fabs(oi * ns - (double)ci) < 1e-3 && fabs(oj * ns - (double)cj) < 1e-3) {
-                const __int128 num = (Mij * ns - (mj * ci + mi * cj)) * ns + Wt * ci * cj;
-                val = to_double(num) / ((double)ns * (double)ns) * down;
-            } else {
-                val = (to_double(Mij) - oi * to_double(mj) - oj * (to_double(mi) - oi * to_double(Wt))) * down;
-            }
-            Mt[(size_t)i * P + j] = val;
-        }
 }
 
 // --------------------------------------------------------------------------- QL iteration
@@ -609,57 +410,265 @@ __global__ void __launch_bounds__(QL_THREADS, 1) snr_ql_kernel(int P, double* __
     for (int i = tid; i < P; i += blockDim.x) sc.d(i) = sm_fail ? NAN : d[i];
 }
 
-// ------------------------------------------------------------------------------- variances
-// q2_k = v_k^T M v_k of 32 eigenvectors (rows of X) per CTA, in e's place.
-__global__ void __launch_bounds__(256) snr_var_kernel(int P, const double* __restrict__ Xws, double* Mws) {
-    constexpr int BR = 32, BJ = 64, BI = 16;
-    __shared__ double As[BI][BR + 1], Bs[BI][BJ];
-    const int t = blockIdx.x, k0 = blockIdx.y * BR, tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+// ------------------------------------------------------------------------- sample pass
+// y_k(x) = sum_i X_ki (O_i(x) - obar_i) for every eigenvector and sample, then the sums over x of Q_k = y_k v_c
+// and |Q_k|^2.  O is a small whole number and X goes in as one (units of 2^-60, two digits of 30 bits), so
+// that y is a sum of whole numbers, exact but for the rounding of X to 2^-61; the mean, subtracted from
+// it in 128 bits, leaves what is small next to O as exact as the rest (directions of small variance, polarised
+// samples), and the one rounding to FP64 comes after it.  The squares are summed as they are: a
+// quadratic form v_k^T M v_k with M = sum_x |v_c|^2 O_c O_c^T takes half the products and, with P^3 FP64
+// ones after them, 11.2 ms where this takes 9.9 (100 trajectories of P = 249, 4096 samples); it cancels as
+// lambda_max / lambda_k, and its sums end at some 1e5 samples (ns^3 2^46 |O|^2 in 128 bits).
+constexpr int WG = 64;         // tile of eigenvectors and of samples
+constexpr int WK = 32;         // parameters per chunk
+constexpr int WGP = WG + 4;    // row of the transposed digits
+constexpr int NSPLIT_MAX = 16; // CTAs that share a tile's samples
+
+// O_k of a sample with spin words word(0 .. W - 1): s_k, s_j s_l, or the sum over a tied group.
+struct OShape {
+    int n, W, P, nu;      // nu: parameters that are single spins or pairs
+    int d, pbc;           // tied distances d + 1 + (k - nu)
+    const int* pairs;     // pairs of the full Jastrow
+    const int* grp_pair;  // tied ansatz: the free groups' pairs (nullptr: parameter n + q is pair q)
+};
+template <class Words>
+__device__ __forceinline__ int o_value(const OShape& o, Words word, int k) {
+    auto bit = [&](int j) { return (int)((word(j >> 6) >> (j & 63)) & 1ull); };
+    if (k < o.n) return 2 * bit(k) - 1;
+    if (k < o.nu) {
+        const int p = o.grp_pair ? __ldg(o.grp_pair + k - o.n) : k - o.n;
+        const int2 jl = __ldg(reinterpret_cast<const int2*>(o.pairs) + p);
+        return 1 - 2 * (bit(jl.x) ^ bit(jl.y));
+    }
+    // all pairs at distance D: (pairs) - 2 (disagreeing ones), from the string shifted by D (rotated
+    // for a ring, where each pair half way round is met twice)
+    const int D = o.d + 1 + k - o.nu, m = o.pbc ? o.n : o.n - D;
+    int dis = 0;
+    for (int q = 0; q < o.W; ++q) {
+        const int left = m - 64 * q;
+        if (left <= 0) break;
+        uint64_t u = 0ull;
+        {
+            const int b = 64 * q + D, i = b >> 6, r = b & 63;
+            if (i < o.W) u = word(i) >> r;
+            if (r && i + 1 < o.W) u |= word(i + 1) << (64 - r);
+        }
+        if (o.pbc) {  // bits n - D and up take the string's first bits
+            const int b = 64 * q - (o.n - D), i = b >> 6, r = b & 63;  // (arithmetic shift: b may be negative)
+            if (i >= 0 && i < o.W) u |= word(i) >> r;
+            if (i + 1 >= 0 && i + 1 < o.W && r) u |= word(i + 1) << (64 - r);
+        }
+        const uint64_t mask = left >= 64 ? ~0ull : (1ull << left) - 1ull;
+        dis += __popcll((word(q) ^ u) & mask);
+    }
+    return o.pbc && 2 * D == o.n ? m / 2 - dis : m - 2 * dis;
+}
+
+// x 2^60 to nearest, |x| < 2 (0 for what is not), in 64-bit integers
+__device__ __forceinline__ long long fix60(double x) {
+    const long long b = __double_as_longlong(x);
+    const int e = (int)((b >> 52) & 0x7FF), sh = 1014 - e;  // mantissa 2^(e - 1075) 2^61
+    const unsigned long long m = ((unsigned long long)b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+    unsigned long long v = sh >= 64 || sh < -9 ? 0ull : sh > 0 ? m >> sh : m << -sh;
+    v = (v + 1) >> 1;
+    return b < 0 ? -(long long)v : (long long)v;
+}
+
+__device__ __forceinline__ double to_double(__int128 v) {  // |v| < 2^116
+    const long long hi = (long long)(v >> 53), lo = (long long)(v - ((__int128)hi << 53));
+    // (hi may take more than 53 bits: then its conversion is the one rounding that counts)
+    return fma((double)hi, 9007199254740992.0, (double)lo);
+}
+
+// What the sample pass takes from the kernel before it and leaves for the one after it, in A's place (the
+// eigenvalues stay in its last rows): 4 P + 2 + 3 P NSPLIT_MAX of its (P - 3) P first doubles.
+struct PassScratch {
+    double* A;
+    int P;
+    __device__ long long* mean_lo() const { return reinterpret_cast<long long*>(A); }          // sum_i X_ki (obar_i -
+    __device__ long long* mean_hi() const { return reinterpret_cast<long long*>(A) + P; }      // o_i) in 2^-60, 128 bits
+    __device__ double* mean_f() const { return A + 2 * P; }                                    // the part of wild obar
+    __device__ long long* o() const { return reinterpret_cast<long long*>(A) + 3 * P; }        // o_i
+    __device__ double* vbar() const { return A + 4 * P; }
+    __device__ double* part(int split) const { return A + 4 * P + 2 + (size_t)split * 3 * P; }  // [3][P]
+};
+
+// Means for the sample pass, 32 eigenvectors per CTA: o_i, the whole number nearest to obar_i (the pass sums
+// O_i - o_i), and the rest of the mean along each eigenvector, from c_i / ns where obar_i = c_i / ns.
+__global__ void __launch_bounds__(256) snr_mean_kernel(int P, int ns, const double2* __restrict__ v,
+                                                       const double* __restrict__ obar, const double* __restrict__ Xws,
+                                                       double* Aws) {
+    const int t = blockIdx.x, k0 = blockIdx.y * 32, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    extern __shared__ __align__(16) double sm[];
+    long long* rf = reinterpret_cast<long long*>(sm);  // [P] obar_i - o_i in units of 2^-60
+    __shared__ double red[8];
+    const PassScratch ps{Aws + (size_t)t * P * P, P};
+    const double* ob = obar + (size_t)t * P;
     const double* X = Xws + (size_t)t * P * P;
-    double* M = Mws + (size_t)t * P * P;
-    double q2[2] = {0.0, 0.0};
-    for (int j0 = 0; j0 < P; j0 += BJ) {
-        double acc[2][4] = {};
-        for (int i0 = 0; i0 < P; i0 += BI) {
-            __syncthreads();
-            for (int e = tid; e < BI * BR; e += 256) {
-                const int r = e / BI, i = e % BI;
-                As[i][r] = (k0 + r < P && i0 + i < P) ? X[(size_t)(k0 + r) * P + i0 + i] : 0.0;
-            }
-            for (int e = tid; e < BI * BJ; e += 256) {
-                // (along the stored row on either side of the diagonal)
-                const bool below = i0 >= j0 + BJ;
-                const int i = below ? e % BI : e / BJ, j = below ? e / BI : e % BJ;
-                const int a = min(i0 + i, j0 + j), b = max(i0 + i, j0 + j);
-                Bs[i][j] = b < P ? M[(size_t)a * P + b] : 0.0;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < BI; ++i)
-#pragma unroll
-                for (int a = 0; a < 2; ++a)
-#pragma unroll
-                    for (int b = 0; b < 4; ++b) acc[a][b] = fma(As[i][2 * ty + a], Bs[i][tx + 16 * b], acc[a][b]);
+    int wild = 0;
+    for (int i = tid; i < P; i += 256) {
+        const double b = ob[i];
+        long long o = 0, r = 0;
+        if (fabs(b) <= 256.0) {
+            o = __double2ll_rn(b);
+            const double c = rint(b * ns);
+            const double f = fabs(b * ns - c) < 1e-3 ? (c - (double)o * ns) / ns : b - (double)o;
+            r = __double2ll_rn(f * 0x1p60);
+        } else {
+            wild = 1;
+        }
+        rf[i] = r;
+        if (k0 == 0) ps.o()[i] = o;
+    }
+    wild = __syncthreads_or(wild);
+    for (int k = k0 + warp; k < min(P, k0 + 32); k += 8) {
+        const double* Xk = X + (size_t)k * P;
+        __int128 s = 0;
+        double f = 0.0;
+        for (int i = lane; i < P; i += 32) {
+            s += (__int128)fix60(Xk[i]) * rf[i];
+            if (wild && !(fabs(ob[i]) <= 256.0)) f = fma(Xk[i], ob[i], f);
         }
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
+        for (int off = 16; off > 0; off >>= 1) {
+            const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)s, off);
+            const long long hi = __shfl_xor_sync(0xffffffffu, (long long)(s >> 64), off);
+            s += ((__int128)hi << 64) + lo;
+            f += __shfl_xor_sync(0xffffffffu, f, off);
+        }
+        s = (s + ((__int128)1 << 59)) >> 60;
+        if (lane == 0) {
+            ps.mean_lo()[k] = (long long)s;
+            ps.mean_hi()[k] = (long long)(s >> 64);
+            ps.mean_f()[k] = f;
+        }
+    }
+    if (k0 > 0) return;
+    const double2* vt = v + (size_t)t * ns;
+    double sx = 0.0, sy = 0.0;
+    for (int x = tid; x < ns; x += 256) {
+        sx += vt[x].x;
+        sy += vt[x].y;
+    }
+    sx = block_sum<8>(sx, red);
+    sy = block_sum<8>(sy, red);
+    if (tid == 0) {
+        ps.vbar()[0] = sx / ns;
+        ps.vbar()[1] = sy / ns;
+    }
+}
+
+// 64 eigenvectors by every nsplit-th tile of 64 samples per CTA, a thread 4 x 4 of a tile.
+__global__ void __launch_bounds__(256, 2) snr_pass_kernel(OShape o, int ns, int nk, int nsplit,
+                                                         const uint64_t* __restrict__ spins,
+                                                         const double2* __restrict__ v,
+                                                         const double* __restrict__ Xws, double* Aws) {
+    const int t = blockIdx.x, k0 = (int)blockIdx.y % nk * WG, split = (int)blockIdx.y / nk;
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, P = o.P, W = o.W;
+    __shared__ __align__(16) int X1[WK][WGP], X0[WK][WGP];  // the digits of X, transposed
+    __shared__ __align__(16) int Os[WK][WG];                // O - o
+    __shared__ uint64_t sw[4][WG];
+    __shared__ double vs[3][WG];                            // v_c and its square
+    __shared__ long long ml[WG], mh[WG];
+    __shared__ double mf[WG];
+    const PassScratch ps{Aws + (size_t)t * P * P, P};
+    const double* X = Xws + (size_t)t * P * P;
+    const double2* vt = v + (size_t)t * ns;
+    const uint64_t* sp = spins + (size_t)t * ns * W;
+    if (tid < WG) {
+        const int k = k0 + tid;
+        ml[tid] = k < P ? ps.mean_lo()[k] : 0;
+        mh[tid] = k < P ? ps.mean_hi()[k] : 0;
+        mf[tid] = k < P ? ps.mean_f()[k] * 0x1p60 : 0.0;
+    }
+    const double vbx = ps.vbar()[0], vby = ps.vbar()[1];
+    double q2[4] = {}, qx[4] = {}, qy[4] = {};
+    for (int x0 = WG * split; x0 < ns; x0 += WG * nsplit) {
+        __syncthreads();
+        for (int e = tid; e < WG * W; e += 256) {
+            const int x = e / W, q = e - x * W;
+            sw[q][x] = x0 + x < ns ? sp[(size_t)(x0 + x) * W + q] : 0ull;
+        }
+        if (tid < WG) {
+            const bool in = x0 + tid < ns;
+            const double a = in ? vt[x0 + tid].x - vbx : 0.0, b = in ? vt[x0 + tid].y - vby : 0.0;
+            vs[0][tid] = a;
+            vs[1][tid] = b;
+            vs[2][tid] = fma(a, a, b * b);
+        }
+        long long a1[4][4], a0[4][4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) a1[a][b] = a0[a][b] = 0;
+        for (int i0 = 0; i0 < P; i0 += WK) {
+            __syncthreads();
+#pragma unroll 2
+            for (int e = tid; e < WK * WG; e += 256) {
+                const int i = e & (WK - 1), r = e / WK;
+                const long long q = k0 + r < P && i0 + i < P ? fix60(X[(size_t)(k0 + r) * P + i0 + i]) : 0ll;
+                X1[i][r] = (int)(q >> 30);
+                X0[i][r] = (int)(q & 0x3FFFFFFF);
+            }
+#pragma unroll 2
+            for (int e = tid; e < WK * WG; e += 256) {
+                const int x = e & (WG - 1), i = e / WG;  // a warp has one parameter
+                int val = 0;
+                if (i0 + i < P)
+                    val = o_value(o, [&](int q) { return sw[q][x]; }, i0 + i) - (int)ps.o()[i0 + i];
+                Os[i][x] = val;
+            }
+            __syncthreads();
+#pragma unroll 4
+            for (int i = 0; i < WK; ++i) {
+                const int4 u1 = *reinterpret_cast<const int4*>(&X1[i][4 * ty]), u0 = *reinterpret_cast<const int4*>(&X0[i][4 * ty]);
+                const int4 ov = *reinterpret_cast<const int4*>(&Os[i][4 * tx]);
+                const int xr[4] = {u1.x, u1.y, u1.z, u1.w}, xl[4] = {u0.x, u0.y, u0.z, u0.w}, oc[4] = {ov.x, ov.y, ov.z, ov.w};
+#pragma unroll
+                for (int a = 0; a < 4; ++a)
+#pragma unroll
+                    for (int b = 0; b < 4; ++b) {
+                        a1[a][b] += (long long)xr[a] * oc[b];
+                        a0[a][b] += (long long)xl[a] * oc[b];
+                    }
+            }
+        }
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            const int r = 4 * ty + a;
+            const __int128 mean = ((__int128)mh[r] << 64) + (unsigned long long)ml[r];
+            const double f = mf[r];
 #pragma unroll
             for (int b = 0; b < 4; ++b) {
-                const int k = k0 + 2 * ty + a, j = j0 + tx + 16 * b;
-                if (k < P && j < P) q2[a] = fma(acc[a][b], X[(size_t)k * P + j], q2[a]);
+                const int x = 4 * tx + b;
+                double y = to_double(((__int128)a1[a][b] << 30) + a0[a][b] - mean);  // in units of 2^-60
+                if (f != 0.0) y -= f;
+                qx[a] = fma(y, vs[0][x], qx[a]);
+                qy[a] = fma(y, vs[1][x], qy[a]);
+                q2[a] = fma(y * y, vs[2][x], q2[a]);
             }
+        }
     }
+    double* part = ps.part(split);
 #pragma unroll
-    for (int a = 0; a < 2; ++a) {
+    for (int a = 0; a < 4; ++a) {
 #pragma unroll
-        for (int off = 8; off > 0; off >>= 1) q2[a] += __shfl_xor_sync(0xffffffffu, q2[a], off);
-        const int k = k0 + 2 * ty + a;
-        if (tx == 0 && k < P) SnrScratch{M, P}.e(k) = q2[a];
+        for (int off = 8; off > 0; off >>= 1) {
+            q2[a] += __shfl_xor_sync(0xffffffffu, q2[a], off);
+            qx[a] += __shfl_xor_sync(0xffffffffu, qx[a], off);
+            qy[a] += __shfl_xor_sync(0xffffffffu, qy[a], off);
+        }
+        const int k = k0 + 4 * ty + a;
+        if (tx == 0 && k < P) {
+            part[k] = q2[a] * 0x1p-120;
+            part[P + k] = qx[a] * 0x1p-60;
+            part[2 * P + k] = qy[a] * 0x1p-60;
+        }
     }
 }
 
 // ------------------------------------------------------------------------------ the solution
-__global__ void __launch_bounds__(256) snr_final_kernel(int P, int ns, const double2* __restrict__ D, double thr,
+__global__ void __launch_bounds__(256) snr_final_kernel(int P, int ns, int nsplit, const double2* __restrict__ D, double thr,
                                                         double eps_svd, double* Aws, const double* __restrict__ Xws,
                                                         double2* __restrict__ delta, double* __restrict__ lam_out) {
     const int t = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -667,7 +676,8 @@ __global__ void __launch_bounds__(256) snr_final_kernel(int P, int ns, const dou
     double2* cf = reinterpret_cast<double2*>(sm);  // [P] filtered coefficients
     __shared__ double red[8];
     const double* X = Xws + (size_t)t * P * P;
-    const SnrScratch sc{Aws + (size_t)t * P * P, P};  // eigenvalue and v^T M v
+    const SnrScratch sc{Aws + (size_t)t * P * P, P};  // eigenvalues
+    const PassScratch ps{Aws + (size_t)t * P * P, P};
     double2* xt = delta + (size_t)t * P;
     const double2* Dt = D + (size_t)t * P;
     double lm = -INFINITY;
@@ -698,9 +708,18 @@ __global__ void __launch_bounds__(256) snr_final_kernel(int P, int ns, const dou
         ax = warp_sum(ax);  // rho_k
         ay = warp_sum(ay);
         if (lane == 0) {
-            const double lam = sc.d(k), r2 = ax * ax + ay * ay;
-            const double var = fmax(sc.e(k) / ns - r2, 0.0);
-            const double snr = sqrt(r2) / sqrt(var / ns + 1e-300);
+            double q2 = 0.0, qx = 0.0, qy = 0.0;
+            for (int p = 0; p < nsplit; ++p) {
+                const double* part = ps.part(p) + k;
+                q2 += part[0];
+                qx += part[P];
+                qy += part[2 * P];
+            }
+            qx /= ns;
+            qy /= ns;
+            const double lam = sc.d(k);
+            const double var = fmax(q2 / ns - (qx * qx + qy * qy), 0.0);
+            const double snr = sqrt(ax * ax + ay * ay) / sqrt(var / ns + 1e-300);
             const double f_snr = 1.0 / (1.0 + pow(thr / snr, 6.0));
             const double f_svd = 1.0 / (1.0 + pow(eps_svd * lm / fmax(lam, 1e-300), 6.0));
             const double inv = lam > 0.0 ? f_snr * f_svd / fmax(lam, 1e-300) : 0.0;
@@ -745,13 +764,14 @@ cudaError_t launch_snr_big(const otvmc_ansatz* a, int ntraj, int ns, const uint6
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(snr_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * P * (int)sizeof(double));
     if (e != cudaSuccess) return e;
-    // (the trajectories along x: a grid's other dimensions end at 65535)
-    const int nt = (P + WG - 1) / WG;
+    // (the trajectories along x: a grid's other dimensions end at 65535.)  The split of the samples does not
+    // depend on the batch, so that neither do the sums.
+    const int nk = (P + WG - 1) / WG, nx = (ns + WG - 1) / WG, nsplit = nx < NSPLIT_MAX ? nx : NSPLIT_MAX;
     snr_tri_kernel<<<ntraj, SNRB_THREADS, smem_tri, s>>>(P, S, Aws, Xws);
-    snr_wgram_kernel<<<dim3(ntraj, nt * (nt + 1) / 2), 256, 0, s>>>(o, ns, spins, v, obar, Aws);
     snr_ql_kernel<<<ntraj, QL_THREADS, smem_ql, s>>>(P, Aws, Xws, status);
-    snr_var_kernel<<<dim3(ntraj, (P + 31) / 32), 256, 0, s>>>(P, Xws, Aws);
-    snr_final_kernel<<<ntraj, 256, 2 * P * (int)sizeof(double), s>>>(P, ns, D, thr, eps_svd, Aws, Xws, delta, lam);
+    snr_mean_kernel<<<dim3(ntraj, (P + 31) / 32), 256, P * (int)sizeof(long long), s>>>(P, ns, v, obar, Xws, Aws);
+    snr_pass_kernel<<<dim3(ntraj, nk * nsplit), 256, 0, s>>>(o, ns, nk, nsplit, spins, v, Xws, Aws);
+    snr_final_kernel<<<ntraj, 256, 2 * P * (int)sizeof(double), s>>>(P, ns, nsplit, D, thr, eps_svd, Aws, Xws, delta, lam);
     count_launch(5);
     return cudaGetLastError();
 }
