@@ -512,7 +512,8 @@ __global__ void __launch_bounds__(256) snr_mean_kernel(int P, int ns, const doub
         if (fabs(b) <= 256.0) {
             o = __double2ll_rn(b);
             const double c = rint(b * ns);
-            const double f = fabs(b * ns - c) < 1e-3 ? (c - (double)o * ns) / ns : b - (double)o;
+            // (c / ns rounded, times ns rounded, is within two roundings of c)
+            const double f = fabs(b * ns - c) <= 0x1p-51 * fabs(c) ? (c - (double)o * ns) / ns : b - (double)o;
             r = __double2ll_rn(f * 0x1p60);
         } else {
             wild = 1;

@@ -143,3 +143,32 @@ def test_more_trajectories_than_a_grid_dimension():
     assert bool((small.abs().amax((1, 2)) > 0).all())
     assert torch.equal(many[-1], small[1])
     assert bool((many[:-1] == small[0]).all())
+
+
+@pytest.mark.parametrize("wild", [False, True])
+def test_obar_that_is_no_column_mean(wild):
+    """The centring takes obar as it is given: not c / ns, and with an entry far beyond any |O|."""
+    n, ns, thr = 14, 700, 1.0
+    ans = _ansatz(abi.OTVMC_JASTROW, n, 0, False)
+    P = ans.P
+    sig = synth.random_spins(5, 1, ns, n)
+    s = sig[0].astype(np.float64)
+    p, q = np.triu_indices(n, 1)
+    O = np.concatenate([s, s[:, p] * s[:, q]], 1)
+    g = np.random.default_rng(9)
+    obar = O.mean(0) + g.normal(0, 0.1, P)
+    if wild:
+        obar[40] = 1000.25
+    v = g.normal(0, 1, ns) + 1j * g.normal(0, 1, ns)
+    Q = np.linalg.qr(g.normal(0, 1, (P, P)))[0]
+    S = (Q * np.linspace(1.0, 2.0, P)) @ Q.T
+    S = 0.5 * (S + S.T)
+    D = g.normal(0, 1, P) + 1j * g.normal(0, 1, P)
+    got = _snr(ans, torch.from_numpy(S[None]).cuda(), torch.from_numpy(obar[None]).cuda(), _pack(sig),
+               to_dev_complex(v[None]), to_dev_complex(D[None]), thr, 1e-12)
+    lam, V = np.linalg.eigh(S)
+    Qx = ((O - obar) @ V) * (v - v.mean())[:, None]
+    var = (np.abs(Qx) ** 2).mean(0) - np.abs(Qx.mean(0)) ** 2
+    rho = V.T @ D
+    want = V @ (rho / lam / (1 + (thr / (np.abs(rho) / np.sqrt(var / ns))) ** 6))
+    assert np.abs(from_dev_complex(got).reshape(P) - want).max() < 1e-10 * np.abs(want).max()
