@@ -26,6 +26,7 @@
 // A and X live in the caller's workspace (2 P^2 doubles per trajectory); the tridiagonal and then the eigenvalues
 // pass from launch to launch in A's last rows (SnrScratch), the sample pass's sums in its first (PassScratch).
 #include "common.cuh"
+#include "rsqrt_pos.cuh"
 
 namespace otvmc {
 
@@ -242,17 +243,6 @@ __global__ void __launch_bounds__(SNRB_THREADS, 1) snr_tri_kernel(int P, const d
 constexpr int QL_THREADS = 384;
 constexpr int QL_APPLY = 288;
 
-// 1 / sqrt(h) for a normal positive h: FP32 approximation y (2^-22) of the root of h's mantissa, then
-// one step of third order, y + y e (1/2 + 3/8 e) with e = 1 - h y^2.
-__device__ __forceinline__ double rsqrt_pos(double h) {
-    const int hw = __double2hiint(h), lw = __double2loint(h);
-    const int E = (hw >> 20) - 1023, k = E >> 1;  // h = mantissa 2^(E & 1) 2^(2 k)
-    const float m = __int_as_float(((127 + (E & 1)) << 23) | ((hw & 0xFFFFF) << 3) | (int)((unsigned)lw >> 29));
-    const int yb = __float_as_int(rsqrtf(m));
-    const double y = __hiloint2double((((yb >> 23) + 896 - k) << 20) | ((yb & 0x7FFFFF) >> 3), yb << 29);
-    const double e = fma(-(h * y), y, 1.0);
-    return fma(y * e, fma(0.375, e, 0.5), y);
-}
 // 2 x for a normal x, and 0 for 0
 __device__ __forceinline__ double twice(double x) {
     const int hw = __double2hiint(x);
