@@ -88,10 +88,8 @@ EvalBufs carve_eval_bufs(Carver& c, const otvmc_ansatz* a, int T, int ns) {
     b.r = c.take<double2>((size_t)T * ns * n);
     b.EH = c.take<double2>((size_t)T * ns * (a->kind == OTVMC_JASTROW ? est_tc_nq(n) : 1));
     b.part_r = c.take<double2>((size_t)T * nblk * n);
-    b.part_sr = c.take<double2>((size_t)T * nblk * n);
     b.part_s = c.take<double>((size_t)T * nblk * n);
     b.mean_r = c.take<double2>((size_t)T * n);
-    b.mean_sr = c.take<double2>((size_t)T * n);
     b.mean_s = c.take<double>((size_t)T * n);
     b.part_v = c.take<double2>((size_t)T * vblk);
     b.part_vmax = c.take<double>((size_t)T * vblk);
@@ -119,10 +117,8 @@ EvalBufs carve_est_bufs(Carver& c, const otvmc_ansatz* a, int T, int ns) {
     b.r = c.take<double2>((size_t)T * ns * n);
     b.EH = c.take<double2>((size_t)T * ns * (a->kind == OTVMC_JASTROW ? est_tc_nq(n) : 1));
     b.part_r = c.take<double2>((size_t)T * nblk * n);
-    b.part_sr = c.take<double2>((size_t)T * nblk * n);
     b.part_s = c.take<double>((size_t)T * nblk * n);
     b.mean_r = c.take<double2>((size_t)T * n);
-    b.mean_sr = c.take<double2>((size_t)T * n);
     b.mean_s = c.take<double>((size_t)T * n);
     b.part_v = c.take<double2>((size_t)T * vblk);
     b.part_vmax = c.take<double>((size_t)T * vblk);

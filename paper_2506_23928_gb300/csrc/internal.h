@@ -115,10 +115,8 @@ struct EvalBufs {
     double2* r;          // [T][ns][n] flip ratios
     double2* EH;         // [T][ns]
     double2* part_r;     // [T][nblk][n]
-    double2* part_sr;    // [T][nblk][n]
     double* part_s;      // [T][nblk][n]
     double2* mean_r;     // [T][n]
-    double2* mean_sr;    // [T][n]
     double* mean_s;      // [T][n]
     double2* part_v;     // [T][vblk]
     double* part_vmax;   // [T][vblk]

@@ -31,10 +31,10 @@
 //     instruction) and commits to an mbarrier;
 //   - epilogue: thread = sample (TMEM lane), in two passes of 8 sites: r_j to global memory
 //     and the sample's E_H over the 16 sites; the ratios also go to shared memory, from which
-//     the per-site sums over the tile's samples (r_j, sigma_j r_j, sigma_j) are taken by
+//     the per-site sums over the tile's samples (r_j, sigma_j) are taken by
 //     eight threads per site and added in a fixed order.
 // E_H leaves as one partial per site block, EHq[t][x][block], summed in order by est2; the
-// per-site sums as one partial per CTA (part_r / part_sr / part_s with est_tc_chunks(ns)
+// per-site sums as one partial per CTA (part_r / part_s with est_tc_chunks(ns)
 // blocks), summed in order by the site-means kernel.  All sums are in a fixed order: the
 // results do not depend on scheduling.
 // Every mbarrier wait is bounded; on timeout the CTA records OTVMC_ERR_TIMEOUT, drains its
@@ -173,7 +173,7 @@ struct Smem {
     uint64_t sw[KB][128];     // the tile's spin words, by 64-site block
     float tab[4][SB];         // aRe, sRe, aJ, sJ of the block's sites
     long long aim[SB];
-    double acc[SB][5];        // per site: sums of Re r, Im r, sigma Re r, sigma Im r, sigma
+    double acc[SB][3];        // per site: sums of Re r, Im r, sigma
 };
 
 // CTAs per SM: by TMEM for KB = 1, by shared memory beyond
@@ -183,7 +183,7 @@ template <int KB>
 __global__ void __launch_bounds__(128, ctas_per_sm(KB)) est_tc_kernel(int n, int ns, double h, const uint64_t* __restrict__ spins,
                                                         const uint8_t* __restrict__ img, SiteTabs tabs,
                                                         float2* __restrict__ r_out, double2* __restrict__ EHq,
-                                                        double2* __restrict__ part_r, double2* __restrict__ part_sr,
+                                                        double2* __restrict__ part_r,
                                                         double* __restrict__ part_s, int nblk, int* status) {
     using namespace tc;
     extern __shared__ uint8_t smem_raw[];
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(128, ctas_per_sm(KB)) est_tc_kernel(int n, int
         S.abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (tid < SB * 5) (&S.acc[0][0])[tid] = 0.0;
+    if (tid < SB * 3) (&S.acc[0][0])[tid] = 0.0;
     if (tid < SB) {
         const size_t o = (size_t)t * nsb * SB + sb * SB + tid;
         S.tab[0][tid] = tabs.aRe[o];
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(128, ctas_per_sm(KB)) est_tc_kernel(int n, int
         if (!*abort_flag) {
             const int u = tid >> 3, p = tid & 7;
             const int sh = (jb0 & 63) + u;
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, a4 = 0.f;
+            float a0 = 0.f, a1 = 0.f, a2 = 0.f;
 #pragma unroll 4
             for (int i = p; i < 128; i += 8) {
                 const float2 r = rs[u][i];
@@ -365,24 +365,18 @@ __global__ void __launch_bounds__(128, ctas_per_sm(KB)) est_tc_kernel(int n, int
                 const float sg = in ? (((S.sw[kw][i] >> sh) & 1ull) ? 1.f : -1.f) : 0.f;
                 a0 += r.x;
                 a1 += r.y;
-                a2 = fmaf(sg, r.x, a2);
-                a3 = fmaf(sg, r.y, a3);
-                a4 += sg;
+                a2 += sg;
             }
 #pragma unroll
             for (int off = 4; off > 0; off >>= 1) {
                 a0 += __shfl_xor_sync(0xffffffffu, a0, off);
                 a1 += __shfl_xor_sync(0xffffffffu, a1, off);
                 a2 += __shfl_xor_sync(0xffffffffu, a2, off);
-                a3 += __shfl_xor_sync(0xffffffffu, a3, off);
-                a4 += __shfl_xor_sync(0xffffffffu, a4, off);
             }
             if (p == 0) {
                 S.acc[u][0] += (double)a0;
                 S.acc[u][1] += (double)a1;
                 S.acc[u][2] += (double)a2;
-                S.acc[u][3] += (double)a3;
-                S.acc[u][4] += (double)a4;
             }
         }
         __syncthreads();  // rs, sw, the sigma tile and TMEM are free again
@@ -392,8 +386,7 @@ __global__ void __launch_bounds__(128, ctas_per_sm(KB)) est_tc_kernel(int n, int
         if (j < n) {
             const size_t o = ((size_t)t * nblk + chunk) * n + j;
             part_r[o] = make_double2(S.acc[tid][0], S.acc[tid][1]);
-            part_sr[o] = make_double2(S.acc[tid][2], S.acc[tid][3]);
-            part_s[o] = S.acc[tid][4];
+            part_s[o] = S.acc[tid][2];
         }
     }
     __syncthreads();
@@ -453,7 +446,7 @@ cudaError_t launch_est_tc(const otvmc_ansatz* a, const uint64_t* spins, int ntra
         e = cudaFuncSetAttribute(etc::est_tc_kernel<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, SM);         \
         if (e != cudaSuccess) return e;                                                                           \
         etc::est_tc_kernel<K><<<grid, 128, SM, s>>>(n, ns, m->h, spins, img, tabs, reinterpret_cast<float2*>(b.r), \
-                                                    b.EH, b.part_r, b.part_sr, b.part_s, nblk, status);           \
+                                                    b.EH, b.part_r, b.part_s, nblk, status);                      \
     } while (0)
     if (KB == 1) OTVMC_EST_TC_LAUNCH(1);
     else OTVMC_EST_TC_LAUNCH(2);

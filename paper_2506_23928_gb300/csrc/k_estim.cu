@@ -65,8 +65,7 @@ __global__ void __launch_bounds__(256) est1_jastrow_kernel(
     int n, int W, int ns, double h, const uint64_t* __restrict__ spins, const long long* __restrict__ Qre,
     const long long* __restrict__ Qim, const long long* __restrict__ base_re, const long long* __restrict__ base_im,
     const long long* __restrict__ QJ, const long long* __restrict__ baseJ, void* __restrict__ r_out,
-    double2* __restrict__ EH_out, double2* __restrict__ part_r, double2* __restrict__ part_sr,
-    double* __restrict__ part_s) {
+    double2* __restrict__ EH_out, double2* __restrict__ part_r, double* __restrict__ part_s) {
     constexpr int SPT = EST_SAMPLES_PER_THREAD;
     const int NT = ((n + 31) / 32) * 32;
     const int SPP = 256 / NT;
@@ -151,13 +150,13 @@ __global__ void __launch_bounds__(256) est1_jastrow_kernel(
     __syncthreads();
 
     const int lane = threadIdx.x & 31, wis = j / 32;  // warp index within the sample's NT threads
-    double2 pr = make_double2(0, 0), psr = make_double2(0, 0);
+    double2 pr = make_double2(0, 0);
     double ps = 0.0;
     if constexpr (FP32T) {
         // MIXED: fields converted from the exact fixed-point sums straight to FP32, the phase
         // reduced modulo 2 pi in fixed point, ratios kept in FP32; per-thread sums in FP32.
         float2* rf = reinterpret_cast<float2*>(r_out);
-        float2 prf = make_float2(0.f, 0.f), psrf = make_float2(0.f, 0.f);
+        float2 prf = make_float2(0.f, 0.f);
         int psi = 0;
         const float bre = active ? fx_to_float(base_re[(size_t)t * n + j]) : 0.f;
         const float bj = active ? fx_to_float(baseJ[j]) : 0.f;
@@ -185,8 +184,6 @@ __global__ void __launch_bounds__(256) est1_jastrow_kernel(
                 fsg = up ? fj : -fj;  // sigma_j f^J_j
                 prf.x += r.x;
                 prf.y += r.y;
-                psrf.x += up ? r.x : -r.x;
-                psrf.y += up ? r.y : -r.y;
                 psi += up ? 1 : -1;
             }
 #pragma unroll
@@ -199,7 +196,6 @@ __global__ void __launch_bounds__(256) est1_jastrow_kernel(
                 ered[sl * (NT / 32) + wis] = make_double2(0.5 * (double)fsg + h * (double)hrx, h * (double)hry);
         }
         pr = make_double2((double)prf.x, (double)prf.y);
-        psr = make_double2((double)psrf.x, (double)psrf.y);
         ps = (double)psi;
     } else {
         double2* rd = reinterpret_cast<double2*>(r_out);
@@ -218,8 +214,6 @@ __global__ void __launch_bounds__(256) est1_jastrow_kernel(
                 contrib = make_double2(0.5 * sj * fj + h * r.x, h * r.y);
                 pr.x += r.x;
                 pr.y += r.y;
-                psr.x += sj * r.x;
-                psr.y += sj * r.y;
                 ps += sj;
             }
             // sum over the sample's sites: butterfly within each warp, then warps in order
@@ -246,28 +240,23 @@ __global__ void __launch_bounds__(256) est1_jastrow_kernel(
     // site sums over this CTA's samples: groups g in order
     __syncthreads();
     double2* red_r = (double2*)qr_s;  // reuse: [SPP][NT]
-    double2* red_sr = red_r + SPP * NT;
-    double* red_s = (double*)(red_sr + SPP * NT);
+    double* red_s = (double*)(red_r + SPP * NT);
     if (g < SPP) {
         red_r[g * NT + j] = pr;
-        red_sr[g * NT + j] = psr;
         red_s[g * NT + j] = ps;
     }
     __syncthreads();
     if (threadIdx.x < n) {
         const int jj = threadIdx.x;
-        double2 a = make_double2(0, 0), b = make_double2(0, 0);
+        double2 a = make_double2(0, 0);
         double c = 0.0;
         for (int gg = 0; gg < SPP; ++gg) {
             a.x += red_r[gg * NT + jj].x;
             a.y += red_r[gg * NT + jj].y;
-            b.x += red_sr[gg * NT + jj].x;
-            b.y += red_sr[gg * NT + jj].y;
             c += red_s[gg * NT + jj];
         }
         const size_t o = ((size_t)t * gridDim.x + blk) * n + jj;
         part_r[o] = a;
-        part_sr[o] = b;
         part_s[o] = c;
     }
 }
@@ -275,7 +264,7 @@ __global__ void __launch_bounds__(256) est1_jastrow_kernel(
 static size_t est1_smem(int n, int W) {
     const int NT = ((n + 31) / 32) * 32, SPP = 256 / NT, SB = SPP * EST_SAMPLES_PER_THREAD;
     size_t a = (size_t)SB * W * 8 + 3 * (size_t)EST_KC * n * 8 + (size_t)SB * (NT / 32) * 16 + 64;
-    size_t b = (size_t)SB * W * 8 + (size_t)SPP * NT * 40 + 64;
+    size_t b = (size_t)SB * W * 8 + (size_t)SPP * NT * 24 + 64;
     return a > b ? a : b;
 }
 
@@ -292,13 +281,13 @@ cudaError_t launch_est1_jastrow(const otvmc_ansatz* a, const uint64_t* spins, in
     if (fp32) {
         cudaFuncSetAttribute(est1_jastrow_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         est1_jastrow_kernel<true><<<grid, 256, smem, s>>>(n, W, ns, m->h, spins, b.Qre, b.Qim, b.base_re, b.base_im,
-                                                         m->QJ_d, m->baseJ_d, b.r, b.EH, b.part_r, b.part_sr,
+                                                         m->QJ_d, m->baseJ_d, b.r, b.EH, b.part_r,
                                                          b.part_s);
     } else {
         cudaFuncSetAttribute(est1_jastrow_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         est1_jastrow_kernel<false><<<grid, 256, smem, s>>>(n, W, ns, m->h, spins, b.Qre, b.Qim, b.base_re,
                                                           b.base_im, m->QJ_d, m->baseJ_d, b.r, b.EH, b.part_r,
-                                                          b.part_sr, b.part_s);
+                                                          b.part_s);
     }
     count_launch();
     return cudaGetLastError();

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(256) est_rbm_kernel(int n, int M, int W, int P
                                                       const long long* __restrict__ QJ,
                                                       const long long* __restrict__ baseJ, double2* __restrict__ r_out,
                                                       double2* __restrict__ EH_out, double2* __restrict__ part_r,
-                                                      double2* __restrict__ part_sr, double* __restrict__ part_s) {
+                                                      double* __restrict__ part_s) {
     constexpr int SPT = EST_SAMPLES_PER_THREAD;
     const int NT = ((n + 31) / 32) * 32;
     const int SPP = 256 / NT;
@@ -167,10 +167,10 @@ __global__ void __launch_bounds__(256) est_rbm_kernel(int n, int M, int W, int P
     double2* ls = gs + SPP * M;           // [SPP][M] lc(gamma)
     double2* ered = ls + SPP * M;         // [SB][NT/32]
     uint64_t* sw = (uint64_t*)(ered + SB * (NT / 32));  // [SPP][W]
-    __shared__ double2 red_r[256], red_sr[256];
+    __shared__ double2 red_r[256];
     __shared__ double red_s[256];
     const RbmTheta th = rbm_split(theta, P, n, M, t);
-    double2 pr = make_double2(0, 0), psr = make_double2(0, 0);
+    double2 pr = make_double2(0, 0);
     double ps = 0.0;
     const int lane = threadIdx.x & 31, wis = j / 32;
     for (int q = 0; q < SPT; ++q) {
@@ -217,8 +217,6 @@ __global__ void __launch_bounds__(256) est_rbm_kernel(int n, int M, int W, int P
             contrib = make_double2(0.5 * sj * fj + h * r.x, h * r.y);
             pr.x += r.x;
             pr.y += r.y;
-            psr.x += sj * r.x;
-            psr.y += sj * r.y;
             ps += sj;
         }
 #pragma unroll
@@ -238,21 +236,18 @@ __global__ void __launch_bounds__(256) est_rbm_kernel(int n, int M, int W, int P
         }
     }
     red_r[threadIdx.x] = pr;
-    red_sr[threadIdx.x] = psr;
     red_s[threadIdx.x] = ps;
     __syncthreads();
     if (threadIdx.x < n) {
         const int jj = threadIdx.x;
-        double2 a = make_double2(0, 0), b = make_double2(0, 0);
+        double2 a = make_double2(0, 0);
         double c = 0.0;
         for (int gg = 0; gg < SPP; ++gg) {
             a = cadd(a, red_r[gg * NT + jj]);
-            b = cadd(b, red_sr[gg * NT + jj]);
             c += red_s[gg * NT + jj];
         }
         const size_t o = ((size_t)t * gridDim.x + blk) * n + jj;
         part_r[o] = a;
-        part_sr[o] = b;
         part_s[o] = c;
     }
 }
@@ -268,7 +263,7 @@ cudaError_t launch_est_rbm(const otvmc_ansatz* a, const double2* theta, const ui
     const otvmc_model* m = a->model;
     dim3 grid(est_blocks(n, ns), ntraj);
     est_rbm_kernel<<<grid, 256, smem, s>>>(n, M, W, (int)a->P, ns, m->h, theta, spins, m->QJ_d, m->baseJ_d, b.r, b.EH,
-                                           b.part_r, b.part_sr, b.part_s);
+                                           b.part_r, b.part_s);
     count_launch();
     return cudaGetLastError();
 }

@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(256) est_rbm_mixed_kernel(int n, int M, int W,
                                                             const float2* __restrict__ atab,
                                                             float2* __restrict__ r_out, double2* __restrict__ EH_out,
                                                             double2* __restrict__ part_r,
-                                                            double2* __restrict__ part_sr, double* __restrict__ part_s) {
+                                                            double* __restrict__ part_s) {
     constexpr int SPT = EST_SAMPLES_PER_THREAD;
     const int NT = ((n + 31) / 32) * 32;
     const int SPP = 256 / NT;
@@ -408,12 +408,12 @@ __global__ void __launch_bounds__(256) est_rbm_mixed_kernel(int n, int M, int W,
     double2* ered = (double2*)(gs + 2 * SPP * M); // [SB][NT/32]
     uint64_t* sw = (uint64_t*)(ered + SB * (NT / 32));  // [SPP][W]
     float2* wf = (float2*)(sw + SPP * W);         // [n][M] W in FP32 (when it fits)
-    __shared__ double2 red_r[256], red_sr[256];
+    __shared__ double2 red_r[256];
     __shared__ double red_s[256];
     const double2* b = theta + (size_t)t * P + n;
     if (WSMEM)
         for (int i = threadIdx.x; i < n * M; i += blockDim.x) wf[i] = wtab[(size_t)t * n * M + i];
-    float2 pr = make_float2(0.f, 0.f), psr = make_float2(0.f, 0.f);
+    float2 pr = make_float2(0.f, 0.f);
     int ps = 0;
     const int lane = threadIdx.x & 31, wis = j / 32;
     for (int q = 0; q < SPT; ++q) {
@@ -473,8 +473,6 @@ __global__ void __launch_bounds__(256) est_rbm_mixed_kernel(int n, int M, int W,
             hry = r.y;
             pr.x += r.x;
             pr.y += r.y;
-            psr.x += up ? r.x : -r.x;
-            psr.y += up ? r.y : -r.y;
             ps += up ? 1 : -1;
         }
 #pragma unroll
@@ -499,23 +497,19 @@ __global__ void __launch_bounds__(256) est_rbm_mixed_kernel(int n, int M, int W,
         }
     }
     red_r[threadIdx.x] = make_double2((double)pr.x, (double)pr.y);
-    red_sr[threadIdx.x] = make_double2((double)psr.x, (double)psr.y);
     red_s[threadIdx.x] = (double)ps;
     __syncthreads();
     if (threadIdx.x < n) {
         const int jj = threadIdx.x;
-        double2 aa = make_double2(0, 0), bb = make_double2(0, 0);
+        double2 aa = make_double2(0, 0);
         double c = 0.0;
         for (int gg = 0; gg < SPP; ++gg) {
             aa.x += red_r[gg * NT + jj].x;
             aa.y += red_r[gg * NT + jj].y;
-            bb.x += red_sr[gg * NT + jj].x;
-            bb.y += red_sr[gg * NT + jj].y;
             c += red_s[gg * NT + jj];
         }
         const size_t o = ((size_t)t * gridDim.x + blk) * n + jj;
         part_r[o] = aa;
-        part_sr[o] = bb;
         part_s[o] = c;
     }
 }
@@ -541,13 +535,13 @@ cudaError_t launch_est_rbm_mixed(const otvmc_ansatz* a, const double2* theta, co
         if (e != cudaSuccess) return e;
         est_rbm_mixed_kernel<true><<<grid, 256, smem, s>>>(n, M, W, (int)a->P, ns, m->h, theta, spins, m->QJ_d,
                                                            m->baseJ_d, tabs.flipT, tabs.w, tabs.a, reinterpret_cast<float2*>(b.r), b.EH, b.part_r,
-                                                           b.part_sr, b.part_s);
+                                                           b.part_s);
     } else {
         e = cudaFuncSetAttribute(est_rbm_mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         est_rbm_mixed_kernel<false><<<grid, 256, smem, s>>>(n, M, W, (int)a->P, ns, m->h, theta, spins, m->QJ_d,
                                                             m->baseJ_d, tabs.flipT, tabs.w, tabs.a, reinterpret_cast<float2*>(b.r), b.EH,
-                                                            b.part_r, b.part_sr, b.part_s);
+                                                            b.part_r, b.part_s);
     }
     count_launch();
     return cudaGetLastError();

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(MAXT, 1) est1_wide_kernel(
     int n, int W, int ns, int nblk, double h, const uint64_t* __restrict__ spins, const float2* __restrict__ rec,
     const long long* __restrict__ Qim, const long long* __restrict__ base_re, const long long* __restrict__ base_im,
     const long long* __restrict__ baseJ, float2* __restrict__ r_out, double2* __restrict__ EH_out,
-    double2* __restrict__ part_r, double2* __restrict__ part_sr, double* __restrict__ part_s) {
+    double2* __restrict__ part_r, double* __restrict__ part_s) {
     const int NT = ((n + 31) / 32) * 32, t = blockIdx.y;
     constexpr int G = EST_G;
     const int g = threadIdx.x / NT, j = threadIdx.x % NT, blk = blockIdx.x * G + g;
@@ -173,7 +173,7 @@ __global__ void __launch_bounds__(MAXT, 1) est1_wide_kernel(
     }
     __syncthreads();  // the table has been read
     const int lane = threadIdx.x & 31, nw = NT / 32;
-    float2 pr = make_float2(0.f, 0.f), psr = make_float2(0.f, 0.f);
+    float2 pr = make_float2(0.f, 0.f);
     int ps = 0;
     const float bre = active ? fx_to_float(base_re[(size_t)t * n + j]) : 0.f;
     const float bj = active ? fx_to_float(baseJ[j]) : 0.f;
@@ -201,8 +201,6 @@ __global__ void __launch_bounds__(MAXT, 1) est1_wide_kernel(
             fsg = up ? fj : -fj;  // sigma_j f^J_j
             pr.x += r.x;
             pr.y += r.y;
-            psr.x += up ? r.x : -r.x;
-            psr.y += up ? r.y : -r.y;
             ps += up ? 1 : -1;
         }
 #pragma unroll
@@ -217,7 +215,6 @@ __global__ void __launch_bounds__(MAXT, 1) est1_wide_kernel(
     if (active) {
         const size_t o = ((size_t)t * nblk + blk) * n + j;
         part_r[o] = make_double2((double)pr.x, (double)pr.y);
-        part_sr[o] = make_double2((double)psr.x, (double)psr.y);
         part_s[o] = (double)ps;
     }
     __syncthreads();
@@ -412,7 +409,7 @@ cudaError_t launch_est1_wide(const otvmc_ansatz* a, const uint64_t* spins, int n
     if (e != cudaSuccess) return e;
     kern<<<dim3((nblk + EST_G - 1) / EST_G, ntraj), EST_G * NT, smem, s>>>(
         n, W, ns, nblk, m->h, spins, rec, b.Qim, b.base_re, b.base_im, m->baseJ_d, reinterpret_cast<float2*>(b.r), b.EH,
-        b.part_r, b.part_sr, b.part_s);
+        b.part_r, b.part_s);
     count_launch(2);
     return cudaGetLastError();
 }
