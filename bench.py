@@ -272,7 +272,6 @@ def rbm_workload(name, stream, fp64_value, steps=3, warmup=2):
     nb = max(abi.otvmc_run_workspace_bytes(ans.handle, desc(k, 0)) for k in range(len(ns_mix)))
     if nb == 0:
         return {"unavailable": "run descriptor rejected"}
-    work = torch.zeros(nb, dtype=torch.uint8, device="cuda")
     g = synth.rng(13)
     batches = []
     for k, (T, ns) in enumerate(zip(counts, ns_mix)):
@@ -282,6 +281,9 @@ def rbm_workload(name, stream, fp64_value, steps=3, warmup=2):
         spins = torch.zeros((T, ns, Wd), dtype=torch.int64, device="cuda")
         check(abi.otvmc_init_chains(ans.handle, T, sum(counts[:k]), ns, seed, spins, stream))
         batches.append((theta, spins))
+    # after the batches: torch may put a tensor of theirs into the rest of the workspace's last 2 MB, which
+    # would keep the whole of it from being given back below
+    work = torch.zeros(nb, dtype=torch.uint8, device="cuda")
     ev = [[torch.cuda.Event(enable_timing=True) for _ in range(len(ns_mix) + 1)] for _ in range(steps)]
     for i in range(warmup + steps):
         marks = ev[i - warmup] if i >= warmup else None
