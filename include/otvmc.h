@@ -247,7 +247,9 @@ OTVMC_API otvmc_status otvmc_local_estimators_noalloc(const otvmc_ansatz* ansatz
  * S = <O^* O> - <O^*><O>, D = <O^* v> - <O^*><v> over the ns samples (definitions after
  * Eq. 8; D = -i F dt + sum_n N^n dW_n by linearity).  Jastrow: O is real (+-1), S real
  * symmetric.
- *   FP64:  S_d [ntraj][P][P] double (full symmetric) from FP64 centred O.
+ *   FP64:  S_d [ntraj][P][P] double (full symmetric), from the exact Gram counts, rounded twice an
+ *          entry (from FP64 centred O where the counts do not fit the workspace of O: more than
+ *          about 1.7 parameters per sample).
  *   MIXED: G_d [ntraj][P][P] float, the uncentred Gram counts sum_x O_xi O_xj for j >= i
  *          (row-major upper triangle; lower part unspecified), from an FP8 (E4M3) tcgen05
  *          GEMM (exact: O = +-1, FP32 accumulation exact below 2^24 samples); obar_d [ntraj][P]
@@ -273,7 +275,9 @@ OTVMC_API otvmc_status otvmc_build_S_F(const otvmc_ansatz* ansatz, const double*
  * not positive definite in the working precision (a pivot not above zero, or a solution that
  * is not finite) the shift is raised (x100, up to 3 times) and OTVMC_ERR_NOT_PD is
  * recorded only if all attempts fail (delta = 0 then).
- *   FP64:  S_d (full FP64), FP64 Cholesky.
+ *   FP64:  S_d (full FP64); P < 48: FP64 Cholesky; beyond, an FP32 Cholesky factor refined to the
+ *          FP64 rounding of the solution with an exact residual, real and imaginary part each, and
+ *          the FP64 Cholesky for trajectories on which FP32 does not decide or converge.
  *   MIXED: G_d + obar_d; tensor-core Cholesky of (S + eps I) / 2^k (2^k the power of two
  *          that bounds the factor's entries by 1; the factor held as two FP16 pieces, 22
  *          significant bits, each 128 x 128 tile product taken as three FP16 tcgen05 products

@@ -493,7 +493,8 @@ static size_t workspace_bytes(const otvmc_ansatz* a, int ntraj, int ns, int prec
     return m + 256;
 }
 
-// A multiple of 256 bytes: clearing 36 GB that end elsewhere takes twice as long.
+// Rounded up to 256 bytes, as the buffers in it are.  (A caller's clearing of 36 GB that end elsewhere was
+// seen to take twice as long.)
 size_t otvmc_workspace_bytes(const otvmc_ansatz* a, int ntraj, int ns, int precision) {
     return (workspace_bytes(a, ntraj, ns, precision) + 255) & ~(size_t)255;
 }
@@ -746,7 +747,7 @@ otvmc_status otvmc_solve_snr(const otvmc_ansatz* a, int ntraj, int ns, const dou
     if (st) return st;
     if (a->kind == OTVMC_RBM) return fail(OTVMC_ERR_UNSUPPORTED, "solve_snr: built for the Jastrow ansaetze");
     if (!snr_big_fits((int)a->P))
-        return fail(OTVMC_ERR_UNSUPPORTED, "solve_snr: P beyond the shared memory of one CTA");
+        return fail(OTVMC_ERR_UNSUPPORTED, "solve_snr: P beyond the filter's bound (about 3000)");
     if (!S_d || !obar_d || !spins_d || !v_d || !D_d || !delta_d || !work_d || !(snr_thresh >= 0.0) ||
         !(eps_svd >= 0.0))
         return fail(OTVMC_ERR_INVALID, "solve_snr: bad arguments");

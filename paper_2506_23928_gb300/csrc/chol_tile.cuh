@@ -1,5 +1,5 @@
 // One-warp Cholesky of a 32 x 32 tile with its inverse, shared by the tensor-core solver's
-// diagonal blocks (k_chol_tc.cu) and the refined FP64 solve (k_solve.cu).
+// diagonal blocks (k_chol_tc.cu) and the refined FP64 solve (k_solve_ref.cu).
 #pragma once
 #include "common.cuh"
 

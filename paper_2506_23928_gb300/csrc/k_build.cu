@@ -450,8 +450,7 @@ cudaError_t launch_D_f64(const otvmc_ansatz* a, const uint64_t* spins, int ntraj
 // integers (below 2^62 while ns |O|^2 < 2^31), so each entry is rounded only when it is converted
 // and when it is divided by ns^2.  One 32 x 32 tile of the upper triangle per CTA, its mirror
 // image written through shared memory.
-template <typename TG>
-__global__ void __launch_bounds__(256) S_counts_kernel(int P, int ns, const TG* __restrict__ G,
+__global__ void __launch_bounds__(256) S_counts_kernel(int P, int ns, const float* __restrict__ G,
                                                        const double* __restrict__ obar, double* __restrict__ S) {
     constexpr int B = 32;
     __shared__ double tile[B][B + 1];
@@ -466,7 +465,7 @@ __global__ void __launch_bounds__(256) S_counts_kernel(int P, int ns, const TG* 
     if (threadIdx.x < B) ci[tx] = I * B + tx < P ? __double2ll_rn(ob[I * B + tx] * ns) : 0ll;
     else if (threadIdx.x < 2 * B) cj[tx] = J * B + tx < P ? __double2ll_rn(ob[J * B + tx] * ns) : 0ll;
     __syncthreads();
-    const TG* Gt = G + (size_t)t * P * P;
+    const float* Gt = G + (size_t)t * P * P;
     double* St = S + (size_t)t * P * P;
     const double den = (double)ns * (double)ns;
 #pragma unroll
@@ -490,7 +489,7 @@ __global__ void __launch_bounds__(256) S_counts_kernel(int P, int ns, const TG* 
 cudaError_t launch_S_counts(int ntraj, int P, int ns, const float* G, const double* obar, double* S, cudaStream_t s) {
     ProfScope prof_(OTVMC_K_SYRK, s);
     const int nt = (P + 31) / 32;
-    S_counts_kernel<float><<<dim3(nt * (nt + 1) / 2, ntraj), 256, 0, s>>>(P, ns, G, obar, S);
+    S_counts_kernel<<<dim3(nt * (nt + 1) / 2, ntraj), 256, 0, s>>>(P, ns, G, obar, S);
     count_launch();
     return cudaGetLastError();
 }

@@ -9,8 +9,8 @@
 // per term with one CTA of eight warps on an SM.  Here a CTA takes as many samples as its threads
 // hold, records of 16 bytes (converted once per trajectory) arrive in chunks of 16 rows by
 // asynchronous copies one chunk ahead, and a record in registers serves several samples.
-// Estimators of 100 x 4096 samples of 160 sites: 8.7 -> 4.06 ms; observables of 64 x 8192 samples of
-// 100 sites: 11.9 -> 4.52 ms (16.5 instructions a term, 72 % of the issue slots).
+// Estimators of 100 x 4096 samples of 160 sites: 8.7 -> 4.04 ms; observables of 64 x 8192 samples of
+// 100 sites: 11.9 -> 4.43 ms (16.5 instructions a term of 32 lanes, padding among them, 72 % of the issue slots).
 #include "common.cuh"
 
 namespace otvmc {
@@ -61,8 +61,8 @@ struct EstSmem {  // byte offsets
 // eight samples is est1_jastrow_kernel's CTA beyond 128 sites, with its partial of the site sums.
 // The real and J fields take every k in order, fma(0 or 1, entry, sum); the imaginary field, whole
 // numbers, takes four k at a time from a table of their 16 partial sums, built per chunk and shared
-// by the CTA's samples.  3.5 instructions a term (predicated additions: 10, bound by the half-rate
-// integer pipe).
+// by the CTA's samples.  7.0 instructions a term of 32 lanes in all (predicated additions: 10.5, bound by
+// the half-rate integer pipe).
 template <int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) est1_wide_kernel(
     int n, int W, int ns, int nblk, double h, const uint64_t* __restrict__ spins, const float2* __restrict__ rec,
